@@ -60,6 +60,8 @@ __global__ void __launch_bounds__(kThreads, 4)
     af_sq_partials_kernel(const float* __restrict__ G, const int8_t* __restrict__ W, bool packed,
                           bool need_csq, int N, int K, float eps1, float* __restrict__ rowpart,
                           float* __restrict__ colpart, unsigned long long* __restrict__ cpart) {
+  dep_wait();
+  dep_trigger();
   __shared__ unsigned long long sh[kThreads / 32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int k0 = blockIdx.x * kColsPerBlock + threadIdx.x * 4;
@@ -126,6 +128,8 @@ __global__ void __launch_bounds__(kThreads)
     af_moments_kernel(const float* __restrict__ rowpart, const float* __restrict__ colpart,
                       int nchunks, int nslabs, int N, int K, int row_blocks, float b2, float omb2,
                       float* __restrict__ R, float* __restrict__ C) {
+  dep_wait();
+  dep_trigger();
   if (static_cast<int>(blockIdx.x) < row_blocks) {
     const int t = blockIdx.x * kThreads + threadIdx.x;
     if (t >= N) return;
@@ -165,6 +169,8 @@ __global__ void __launch_bounds__(kThreads)
 __global__ void __launch_bounds__(kThreads)
     af_factors_kernel(const float* __restrict__ R, const float* __restrict__ C, int N, int K,
                       float* __restrict__ a, float* __restrict__ b, float* __restrict__ scal) {
+  dep_wait();
+  dep_trigger();
   __shared__ double shd[kThreads / 32];
   __shared__ float rbar_s;
   double rs = 0.0;
@@ -190,6 +196,8 @@ __device__ __forceinline__ float af_u(float g, float an, float bk) {
 __global__ void __launch_bounds__(kThreads)
     af_usq_partials_kernel(const float* __restrict__ G, const float* __restrict__ a,
                            const float* __restrict__ b, int N, int K, float* __restrict__ upart) {
+  dep_wait();
+  dep_trigger();
   __shared__ float sh[kThreads / 32];
   const int k0 = blockIdx.x * kColsPerBlock + threadIdx.x * 4;
   const int n0 = blockIdx.y * kRowsPerSlab;
@@ -228,6 +236,8 @@ __global__ void __launch_bounds__(kThreads)
                        const unsigned long long* __restrict__ cpart, int nparts, float s_w,
                        float rho, float eps2, float clip_d, int scale_parameter,
                        float weight_decay, float* __restrict__ out) {
+  dep_wait();
+  dep_trigger();
   __shared__ double shd[kThreads / 32];
   __shared__ unsigned long long shu[kThreads / 32];
   double us = 0.0;
@@ -265,6 +275,8 @@ __global__ void __launch_bounds__(kThreads)
                     const float* __restrict__ fa, const float* __restrict__ fb,
                     const float* __restrict__ scal, int N, int K, const ApplyArgs a,
                     unsigned long long* changed) {
+  dep_wait();
+  dep_trigger();
   const float step = scal[1], decay = scal[2];
   const int64_t ngroups = (static_cast<int64_t>(N) * K) >> 2;  // K % 4 == 0: no ragged group
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
@@ -365,18 +377,22 @@ int launch_adafactor_stats(const float* G, const int8_t* W, bool packed, float s
   float* scal = scalars_out;
   const int n = static_cast<int>(N), k = static_cast<int>(K);
   const dim3 grid(L.gx, L.nslabs);
-  af_sq_partials_kernel<<<grid, kThreads, 0, stream>>>(G, W, packed, h.scale_parameter != 0, n, k,
-                                                       h.eps1, rowpart, colpart, cpart);
+  if (launch_dep(af_sq_partials_kernel, grid, kThreads, 0, stream, G, W, packed,
+                 h.scale_parameter != 0, n, k, h.eps1, rowpart, colpart, cpart))
+    return 3;
   const int row_blocks = (n + kThreads - 1) / kThreads;
   const int col_blocks = (k + 31) / 32;
-  af_moments_kernel<<<row_blocks + col_blocks, kThreads, 0, stream>>>(
-      rowpart, colpart, L.nchunks, L.nslabs, n, k, row_blocks, h.b2, h.omb2, R, C);
-  af_factors_kernel<<<(n + k + kThreads - 1) / kThreads, kThreads, 0, stream>>>(R, C, n, k, a_out,
-                                                                              b_out, scal);
-  af_usq_partials_kernel<<<grid, kThreads, 0, stream>>>(G, a_out, b_out, n, k, upart);
-  af_finalize_kernel<<<1, kThreads, 0, stream>>>(n, k, upart, cpart, L.nparts, s_w, h.rho, h.eps2,
-                                             h.clip_d, h.scale_parameter, h.weight_decay, scal);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  if (launch_dep(af_moments_kernel, row_blocks + col_blocks, kThreads, 0, stream, rowpart, colpart,
+                 L.nchunks, L.nslabs, n, k, row_blocks, h.b2, h.omb2, R, C))
+    return 3;
+  if (launch_dep(af_factors_kernel, (n + k + kThreads - 1) / kThreads, kThreads, 0, stream, R, C,
+                 n, k, a_out, b_out, scal))
+    return 3;
+  if (launch_dep(af_usq_partials_kernel, grid, kThreads, 0, stream, G, a_out, b_out, n, k,
+                 upart))
+    return 3;
+  return launch_dep(af_finalize_kernel, 1, kThreads, 0, stream, n, k, upart, cpart, L.nparts, s_w,
+                    h.rho, h.eps2, h.clip_d, h.scale_parameter, h.weight_decay, scal);
 }
 
 int launch_adafactor_apply(const float* G, int8_t* W, bool packed, const float* fa,
@@ -399,12 +415,11 @@ int launch_adafactor_apply(const float* G, int8_t* W, bool packed, const float* 
   if (blocks > static_cast<int64_t>(sms) * 8) blocks = static_cast<int64_t>(sms) * 8;
   if (blocks < 1) blocks = 1;
   if (N * K >= (int64_t(1) << 32))
-    af_apply_kernel<true><<<static_cast<int>(blocks), kThreads, 0, stream>>>(
-        G, W, packed, fa, fb, scalars, static_cast<int>(N), static_cast<int>(K), a, changed);
-  else
-    af_apply_kernel<false><<<static_cast<int>(blocks), kThreads, 0, stream>>>(
-        G, W, packed, fa, fb, scalars, static_cast<int>(N), static_cast<int>(K), a, changed);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+    return launch_dep(af_apply_kernel<true>, static_cast<int>(blocks), kThreads, 0, stream, G, W,
+                      packed, fa, fb, scalars, static_cast<int>(N), static_cast<int>(K), a,
+                      changed);
+  return launch_dep(af_apply_kernel<false>, static_cast<int>(blocks), kThreads, 0, stream, G, W,
+                    packed, fa, fb, scalars, static_cast<int>(N), static_cast<int>(K), a, changed);
 }
 
 }  // namespace dqt

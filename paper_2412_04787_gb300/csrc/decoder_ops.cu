@@ -38,6 +38,8 @@ template <bool INV>
 __global__ void __launch_bounds__(kRopeThreads)
     rope_kernel(const uint4* __restrict__ x, uint4* __restrict__ y, const float4* __restrict__ cs,
                 int64_t nvec, int64_t row_vecs, int64_t S, int64_t head_vecs) {
+  dep_wait();
+  dep_trigger();
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kRopeThreads;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * kRopeThreads + threadIdx.x; i < nvec;
        i += stride) {
@@ -97,6 +99,8 @@ __device__ __forceinline__ void lse_block(float& m, float& s, float* sh_m, float
 __global__ void __launch_bounds__(kCeThreads)
     ce_fwd_kernel(const uint4* __restrict__ logits, const int64_t* __restrict__ tgt, int64_t V,
                   float* __restrict__ lse, float* __restrict__ row_loss) {
+  dep_wait();
+  dep_trigger();
   __shared__ float sh_m[kCeThreads / 32], sh_s[kCeThreads / 32];
   const int64_t r = blockIdx.x;
   const int64_t nv = V >> 3;
@@ -138,6 +142,8 @@ __global__ void __launch_bounds__(kCeThreads)
     ce_bwd_kernel(const uint4* __restrict__ logits, const int64_t* __restrict__ tgt,
                   const float* __restrict__ lse, const float* __restrict__ scale, int64_t V,
                   uint4* __restrict__ dlogits) {
+  dep_wait();
+  dep_trigger();
   const int64_t r = blockIdx.x;
   const int64_t nv = V >> 3;
   const int64_t t = tgt[r];
@@ -177,6 +183,8 @@ constexpr int kEwThreads = 256;
 __global__ void __launch_bounds__(kEwThreads)
     swiglu_kernel(const uint4* __restrict__ g, const uint4* __restrict__ u, uint4* __restrict__ h,
                   int64_t nvec) {
+  dep_wait();
+  dep_trigger();
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kEwThreads;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * kEwThreads + threadIdx.x; i < nvec;
        i += stride) {
@@ -199,6 +207,8 @@ __global__ void __launch_bounds__(kEwThreads)
     swiglu_bwd_kernel(const uint4* __restrict__ g, const uint4* __restrict__ u,
                       const uint4* __restrict__ dh, uint4* __restrict__ dg,
                       uint4* __restrict__ du, int64_t nvec) {
+  dep_wait();
+  dep_trigger();
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kEwThreads;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * kEwThreads + threadIdx.x; i < nvec;
        i += stride) {
@@ -234,6 +244,8 @@ template <int VPL>
 __global__ void __launch_bounds__(32 * kNormWarps)
     rmsnorm_fwd_kernel(const uint4* __restrict__ x, const uint4* __restrict__ w, float eps,
                        int64_t rows, int nv, uint4* __restrict__ y, float* __restrict__ rstd) {
+  dep_wait();
+  dep_trigger();
   const int lane = threadIdx.x & 31;
   const int64_t row = static_cast<int64_t>(blockIdx.x) * kNormWarps + (threadIdx.x >> 5);
   if (row >= rows) return;
@@ -281,6 +293,8 @@ __global__ void __launch_bounds__(32 * kNormWarps)
     rmsnorm_bwd_kernel(const uint4* __restrict__ x, const uint4* __restrict__ w,
                        const float* __restrict__ rstd, const uint4* __restrict__ dy, int64_t rows,
                        int nv, uint4* __restrict__ dx, float* __restrict__ part) {
+  dep_wait();
+  dep_trigger();
   const int lane = threadIdx.x & 31;
   const int64_t wid = static_cast<int64_t>(blockIdx.x) * kNormWarps + (threadIdx.x >> 5);
   const int64_t nwarps = static_cast<int64_t>(gridDim.x) * kNormWarps;
@@ -350,6 +364,8 @@ __global__ void __launch_bounds__(32 * kNormWarps)
 // in increasing p, and the block adds the 8 warp sums in warp order.
 __global__ void __launch_bounds__(256)
     rmsnorm_dw_kernel(const float* __restrict__ part, int64_t P, int D, uint16_t* __restrict__ dw) {
+  dep_wait();
+  dep_trigger();
   __shared__ float sh[8][33];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int col = blockIdx.x * 32 + lane;
@@ -395,45 +411,41 @@ int launch_rope(const uint16_t* x, uint16_t* y, const float* cos_sin, int64_t ro
   auto* yv = reinterpret_cast<uint4*>(y);
   auto* cv = reinterpret_cast<const float4*>(cos_sin);
   if (inverse)
-    rope_kernel<true><<<blocks, kRopeThreads, 0, stream>>>(xv, yv, cv, nvec, row_vecs, S, head_vecs);
-  else
-    rope_kernel<false><<<blocks, kRopeThreads, 0, stream>>>(xv, yv, cv, nvec, row_vecs, S, head_vecs);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+    return launch_dep(rope_kernel<true>, blocks, kRopeThreads, 0, stream, xv, yv, cv, nvec,
+                      row_vecs, S, head_vecs);
+  return launch_dep(rope_kernel<false>, blocks, kRopeThreads, 0, stream, xv, yv, cv, nvec, row_vecs,
+                    S, head_vecs);
 }
 
 int launch_ce_fwd(const uint16_t* logits, const int64_t* targets, int64_t M, int64_t V,
                   float* lse, float* row_loss, cudaStream_t stream) {
-  ce_fwd_kernel<<<static_cast<unsigned>(M), kCeThreads, 0, stream>>>(
-      reinterpret_cast<const uint4*>(logits), targets, V, lse, row_loss);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(ce_fwd_kernel, static_cast<unsigned>(M), kCeThreads, 0, stream,
+                    reinterpret_cast<const uint4*>(logits), targets, V, lse, row_loss);
 }
 
 int launch_ce_bwd(const uint16_t* logits, const int64_t* targets, const float* lse,
                   const float* scale, int64_t M, int64_t V, uint16_t* dlogits,
                   cudaStream_t stream) {
-  ce_bwd_kernel<<<static_cast<unsigned>(M), kCeThreads, 0, stream>>>(
-      reinterpret_cast<const uint4*>(logits), targets, lse, scale, V,
-      reinterpret_cast<uint4*>(dlogits));
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(ce_bwd_kernel, static_cast<unsigned>(M), kCeThreads, 0, stream,
+                    reinterpret_cast<const uint4*>(logits), targets, lse, scale, V,
+                    reinterpret_cast<uint4*>(dlogits));
 }
 
 int launch_swiglu(const uint16_t* g, const uint16_t* u, uint16_t* h, int64_t n,
                   cudaStream_t stream) {
   const int64_t nvec = n / 8;
-  swiglu_kernel<<<grid_cap(nvec, kEwThreads), kEwThreads, 0, stream>>>(
-      reinterpret_cast<const uint4*>(g), reinterpret_cast<const uint4*>(u),
-      reinterpret_cast<uint4*>(h), nvec);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(swiglu_kernel, grid_cap(nvec, kEwThreads), kEwThreads, 0, stream,
+                    reinterpret_cast<const uint4*>(g), reinterpret_cast<const uint4*>(u),
+                    reinterpret_cast<uint4*>(h), nvec);
 }
 
 int launch_swiglu_bwd(const uint16_t* g, const uint16_t* u, const uint16_t* dh, uint16_t* dg,
                       uint16_t* du, int64_t n, cudaStream_t stream) {
   const int64_t nvec = n / 8;
-  swiglu_bwd_kernel<<<grid_cap(nvec, kEwThreads), kEwThreads, 0, stream>>>(
-      reinterpret_cast<const uint4*>(g), reinterpret_cast<const uint4*>(u),
-      reinterpret_cast<const uint4*>(dh), reinterpret_cast<uint4*>(dg),
-      reinterpret_cast<uint4*>(du), nvec);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(swiglu_bwd_kernel, grid_cap(nvec, kEwThreads), kEwThreads, 0, stream,
+                    reinterpret_cast<const uint4*>(g), reinterpret_cast<const uint4*>(u),
+                    reinterpret_cast<const uint4*>(dh), reinterpret_cast<uint4*>(dg),
+                    reinterpret_cast<uint4*>(du), nvec);
 }
 
 size_t rmsnorm_bwd_ws(int64_t rows, int64_t D) {
@@ -448,10 +460,9 @@ static int rms_launch(const uint16_t* x, const uint16_t* w, float eps, int64_t r
                       uint16_t* y, float* rstd, cudaStream_t stream) {
   const int nv = static_cast<int>(D / 8);
   const unsigned blocks = static_cast<unsigned>((rows + kNormWarps - 1) / kNormWarps);
-  rmsnorm_fwd_kernel<VPL><<<blocks, 32 * kNormWarps, 0, stream>>>(
-      reinterpret_cast<const uint4*>(x), reinterpret_cast<const uint4*>(w), eps, rows, nv,
-      reinterpret_cast<uint4*>(y), rstd);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(rmsnorm_fwd_kernel<VPL>, blocks, 32 * kNormWarps, 0, stream,
+                    reinterpret_cast<const uint4*>(x), reinterpret_cast<const uint4*>(w), eps,
+                    rows, nv, reinterpret_cast<uint4*>(y), rstd);
 }
 
 template <int VPL>
@@ -462,13 +473,14 @@ static int rms_bwd_launch(const uint16_t* x, const uint16_t* w, const float* rst
   const int64_t need = (rows + kNormWarps - 1) / kNormWarps;
   const int64_t sms = norm_blocks_bwd();
   const unsigned blocks = static_cast<unsigned>(sms < need ? sms : need);
-  rmsnorm_bwd_kernel<VPL><<<blocks, 32 * kNormWarps, 0, stream>>>(
-      reinterpret_cast<const uint4*>(x), reinterpret_cast<const uint4*>(w), rstd,
-      reinterpret_cast<const uint4*>(dy), rows, nv, reinterpret_cast<uint4*>(dx), part);
+  if (launch_dep(rmsnorm_bwd_kernel<VPL>, blocks, 32 * kNormWarps, 0, stream,
+                 reinterpret_cast<const uint4*>(x), reinterpret_cast<const uint4*>(w), rstd,
+                 reinterpret_cast<const uint4*>(dy), rows, nv, reinterpret_cast<uint4*>(dx),
+                 part))
+    return 3;
   const int64_t P = static_cast<int64_t>(blocks) * kNormWarps;
-  rmsnorm_dw_kernel<<<static_cast<unsigned>((D + 31) / 32), 256, 0, stream>>>(
-      part, P, static_cast<int>(D), dw);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(rmsnorm_dw_kernel, static_cast<unsigned>((D + 31) / 32), 256, 0, stream, part,
+                    P, static_cast<int>(D), dw);
 }
 
 int launch_rmsnorm(const uint16_t* x, const uint16_t* w, float eps, int64_t rows, int64_t D,

@@ -94,6 +94,21 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64
 }
 
 // ---------------------------------------------------------------------------
+// Programmatic dependent launch (launch_dep in dqt_internal.h): the next
+// kernel of the stream may start while this one runs.  A kernel launched so
+// calls dep_wait in every thread before its first access to global memory:
+// it returns when the kernels before it have finished and their writes are
+// visible.  Since each kernel waits for its predecessor, a kernel that has
+// waited has all earlier work behind it.  dep_trigger lets the next kernel's
+// blocks take the SM resources this one leaves free, or frees early, and run
+// their set-up (barriers, tensor memory, descriptors) up to their own wait.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dep_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// ---------------------------------------------------------------------------
 // Thread-block clusters (pairs of CTAs on the two SMs of a TPC).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t cluster_ctarank() {

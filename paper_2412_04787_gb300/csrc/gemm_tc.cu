@@ -645,7 +645,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&acc_empty[b], kEpiWarps);
     }
     mbar_init(drain_bar, 1);
-    if (EPI == GEMM_DW) *uc_s = p.uc_dev ? *p.uc_dev : p.uc;
+    if (EPI == GEMM_DW) {
+      dep_wait();
+      *uc_s = p.uc_dev ? *p.uc_dev : p.uc;
+    }
     fence_mbarrier_init();
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
@@ -655,6 +658,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  dep_wait();
+  dep_trigger();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -911,6 +916,7 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
   // The dynamic shared window is 1024-byte aligned in practice; if it is not
   // and the slack cannot absorb it, every CTA of the grid returns here alike.
   if (((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u) > static_cast<uint32_t>(S::SLACK)) {
+    dep_wait();
     if (threadIdx.x == 0) record_timeout(p.status);
     return;
   }
@@ -943,7 +949,10 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
       mbar_init(&acc_empty[b], 2 * EW);
     }
     mbar_init(drain_bar, 1);
-    if (EPI == GEMM_DW && UCD) *uc_s = *p.uc_dev;
+    if (EPI == GEMM_DW && UCD) {
+      dep_wait();
+      *uc_s = *p.uc_dev;
+    }
     fence_mbarrier_init();
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
@@ -960,6 +969,8 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
   const uint32_t tmem = *tmem_slot;
   const uint32_t full_lead = mapa_shared(smem_u32(full), 0);
   const uint32_t acc_empty_lead = mapa_shared(smem_u32(acc_empty), 0);
+  dep_wait();
+  dep_trigger();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -1417,8 +1428,7 @@ int launch_tiles(const CUtensorMap& ta, const CUtensorMap& tb, Params p, cudaStr
   p.num_n = (p.N + BN - 1) / BN;
   p.num_tiles = ((p.M + BM - 1) / BM) * p.num_n;
   const int grid = p.num_tiles < sms ? p.num_tiles : sms;
-  kern<<<grid, kThreads, smem, stream>>>(ta, tb, p);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(kern, grid, kThreads, smem, stream, ta, tb, p);
 }
 
 template <bool A_MN, bool B_MN, int EPI, bool PK = false, bool DR = false, bool UCD = false>
@@ -1527,16 +1537,18 @@ int launch_pairs(const CUtensorMap& ta, const CUtensorMap& tb, Params p, cudaStr
   static int max_clusters = 0;  // per template instance
   pair_tiling(p, EPI == GEMM_DW);
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_dep
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.blockDim = dim3(threads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   if (max_clusters == 0) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
         cudaSuccess)
@@ -1546,7 +1558,9 @@ int launch_pairs(const CUtensorMap& ta, const CUtensorMap& tb, Params p, cudaStr
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cfg.gridDim = dim3(sms, 1, 1);
     int n = 0;
+    cfg.numAttrs = 1;  // the cluster shape
     if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) return 3;
+    cfg.numAttrs = 2;
     max_clusters = n;
   }
   p.full_units = p.num_tiles;
@@ -1815,16 +1829,18 @@ int launch_dw_group(const GemmLaunch& g0, const GemmLaunch& g1, cudaStream_t str
   constexpr int threads = PairCfg<GEMM_DW, false>::THREADS;
   static int max_clusters = 0;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see launch_dep
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.blockDim = dim3(threads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   if (max_clusters == 0) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
         cudaSuccess)
@@ -1834,7 +1850,9 @@ int launch_dw_group(const GemmLaunch& g0, const GemmLaunch& g1, cudaStream_t str
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cfg.gridDim = dim3(sms, 1, 1);
     int n = 0;
+    cfg.numAttrs = 1;  // the cluster shape
     if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) return 3;
+    cfg.numAttrs = 2;
     max_clusters = n;
   }
   const int total = p[0].num_tiles + p[1].num_tiles;

@@ -32,6 +32,8 @@ __device__ __forceinline__ uint32_t pack_word(uint32_t w) {  // 4 int8 codes -> 
 
 __global__ void __launch_bounds__(kThreads)
     pack_kernel(const int8_t* __restrict__ c, int64_t n, uint8_t* __restrict__ out) {
+  dep_wait();
+  dep_trigger();
   const int64_t nvec = n >> 4;  // 16 codes -> one 32-bit word of 4 bytes
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < nvec;
@@ -52,6 +54,8 @@ __global__ void __launch_bounds__(kThreads)
 
 __global__ void __launch_bounds__(kThreads)
     unpack_kernel(const uint8_t* __restrict__ p, int64_t n, int8_t* __restrict__ c) {
+  dep_wait();
+  dep_trigger();
   const int64_t nvec = n >> 4;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < nvec;
@@ -87,6 +91,8 @@ __device__ __forceinline__ uint32_t tern_e4m3(uint32_t f) {
 
 __global__ void __launch_bounds__(kThreads)
     packed_to_bf16_kernel(const uint8_t* __restrict__ p, int64_t n, uint16_t* __restrict__ img) {
+  dep_wait();
+  dep_trigger();
   const int64_t nvec = n >> 4;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < nvec;
@@ -107,6 +113,8 @@ __global__ void __launch_bounds__(kThreads)
 
 __global__ void __launch_bounds__(kThreads)
     packed_to_fp8_kernel(const uint8_t* __restrict__ p, int64_t n, uint8_t* __restrict__ out) {
+  dep_wait();
+  dep_trigger();
   const int64_t nvec = n >> 4;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < nvec;
@@ -128,23 +136,19 @@ __global__ void __launch_bounds__(kThreads)
 }  // namespace
 
 int launch_pack_ternary(const int8_t* c, int64_t n, uint8_t* out, cudaStream_t stream) {
-  pack_kernel<<<blocks_for(n >> 4), kThreads, 0, stream>>>(c, n, out);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(pack_kernel, blocks_for(n >> 4), kThreads, 0, stream, c, n, out);
 }
 
 int launch_unpack_ternary(const uint8_t* p, int64_t n, int8_t* c, cudaStream_t stream) {
-  unpack_kernel<<<blocks_for(n >> 4), kThreads, 0, stream>>>(p, n, c);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(unpack_kernel, blocks_for(n >> 4), kThreads, 0, stream, p, n, c);
 }
 
 int launch_packed_to_bf16(const uint8_t* p, int64_t n, uint16_t* img, cudaStream_t stream) {
-  packed_to_bf16_kernel<<<blocks_for(n >> 4), kThreads, 0, stream>>>(p, n, img);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(packed_to_bf16_kernel, blocks_for(n >> 4), kThreads, 0, stream, p, n, img);
 }
 
 int launch_packed_to_fp8(const uint8_t* p, int64_t n, uint8_t* out, cudaStream_t stream) {
-  packed_to_fp8_kernel<<<blocks_for(n >> 4), kThreads, 0, stream>>>(p, n, out);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(packed_to_fp8_kernel, blocks_for(n >> 4), kThreads, 0, stream, p, n, out);
 }
 
 }  // namespace dqt

@@ -72,6 +72,8 @@ __global__ void __launch_bounds__(kAqWarps * 32)
     act_quant_kernel(const uint16_t* __restrict__ X, int T, int K, int8_t* __restrict__ Xq,
                      float* __restrict__ s_x, uint16_t* __restrict__ Xq_img,
                      uint16_t* __restrict__ Xdq) {
+  dep_wait();
+  dep_trigger();
   const int row = blockIdx.x * kAqWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= T) return;
@@ -263,6 +265,8 @@ __global__ void __launch_bounds__(32 * 17, 1)
   const int lane = threadIdx.x & 31;
   ring.init_barriers();
   __syncthreads();
+  dep_wait();
+  dep_trigger();
   if (warp == 0) {
     if (lane == 0) ring.produce(reinterpret_cast<const uint8_t*>(X), status, limit_ns);
     return;
@@ -369,6 +373,8 @@ __global__ void __launch_bounds__(32 * 17, 1)
   const int lane = threadIdx.x & 31;
   ring.init_barriers();
   __syncthreads();
+  dep_wait();
+  dep_trigger();
   if (warp == 0) {
     if (lane == 0) ring.produce(reinterpret_cast<const uint8_t*>(Xq), status, limit_ns);
     return;
@@ -421,6 +427,8 @@ __global__ void __launch_bounds__(32 * 17, 1)
 __global__ void __launch_bounds__(256)
     codes_to_xdq_kernel(const int8_t* __restrict__ Xq, const float* __restrict__ s_x, int T,
                         int K, uint16_t* __restrict__ Xdq) {
+  dep_wait();
+  dep_trigger();
   __shared__ uint16_t table[8][256];
   const int wid = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -472,6 +480,8 @@ __device__ __forceinline__ void codes16_to_bf16(const uint4 u, uint4& o0, uint4&
 
 __global__ void codes_to_bf16_kernel(const int8_t* __restrict__ W, int64_t numel,
                                      uint16_t* __restrict__ img) {
+  dep_wait();
+  dep_trigger();
   const int64_t nvec = numel >> 4;  // 16-code vectors
   const int64_t nthr = static_cast<int64_t>(gridDim.x) * blockDim.x;
   const uint4* src = reinterpret_cast<const uint4*>(W);
@@ -514,6 +524,8 @@ __device__ __forceinline__ uint32_t codes4_to_e4m3(uint32_t w) {
 
 __global__ void codes_to_fp8_kernel(const int8_t* __restrict__ W, int64_t numel,
                                     uint8_t* __restrict__ out) {
+  dep_wait();
+  dep_trigger();
   const int64_t nvec = numel >> 4;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   const uint4* src = reinterpret_cast<const uint4*>(W);
@@ -536,6 +548,8 @@ __global__ void codes_to_fp8_kernel(const int8_t* __restrict__ W, int64_t numel,
 // 16 h of its K codes, then their l.  One thread step: 16 codes of a row.
 __global__ void codes_to_fp8_split_kernel(const int8_t* __restrict__ W, int64_t N, int64_t K,
                                           uint8_t* __restrict__ out) {
+  dep_wait();
+  dep_trigger();
   const int64_t vpr = K >> 4;  // 16-code vectors per row
   const int64_t nvec = N * vpr;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
@@ -660,8 +674,8 @@ int launch_ring(Kern kern, bool& attr_set, int64_t T, int rpc, int W, int S, int
   const int blocks = static_cast<int>(T < sms ? T : sms);
   const size_t smem =
       static_cast<size_t>(S) * rpc * row_bytes + 16 * static_cast<size_t>(S) + 512 * W;
-  kern<<<blocks, 32 * (W + 1), smem, stream>>>(args..., S, W, rpc, status, wait_limit_ns());
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(kern, blocks, 32 * (W + 1), smem, stream, args..., S, W, rpc, status,
+                    wait_limit_ns());
 }
 
 // Rows staged in shared memory when at least four fit in the ring; -1 when
@@ -685,9 +699,8 @@ int launch_aq(const uint16_t* X, int64_t T, int64_t K, int8_t* Xq, float* s_x, u
   }
   // rows longer than 48 KB (K > 24576): one warp per row, two passes
   const int blocks = static_cast<int>((T + kAqWarps - 1) / kAqWarps);
-  act_quant_kernel<F8><<<blocks, kAqWarps * 32, 0, stream>>>(X, static_cast<int>(T),
-                                                            static_cast<int>(K), Xq, s_x, Xq_img, Xdq);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(act_quant_kernel<F8>, blocks, kAqWarps * 32, 0, stream, X, static_cast<int>(T),
+                    static_cast<int>(K), Xq, s_x, Xq_img, Xdq);
 }
 
 }  // namespace
@@ -712,9 +725,8 @@ int launch_codes_to_xdq(const int8_t* Xq, const float* s_x, int64_t T, int64_t K
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t want = (T + 7) / 8;
   const int blocks = static_cast<int>(want < 4 * sms ? want : 4 * sms);
-  codes_to_xdq_kernel<<<blocks, 256, 0, stream>>>(Xq, s_x, static_cast<int>(T),
-                                                  static_cast<int>(K), Xdq);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(codes_to_xdq_kernel, blocks, 256, 0, stream, Xq, s_x, static_cast<int>(T),
+                    static_cast<int>(K), Xdq);
 }
 
 int launch_act_quant_fp8(const uint16_t* X, int64_t T, int64_t K, uint8_t* Xq8, float* s8,
@@ -724,21 +736,21 @@ int launch_act_quant_fp8(const uint16_t* X, int64_t T, int64_t K, uint8_t* Xq8, 
 
 int launch_codes_to_fp8(const int8_t* W, int64_t numel, uint8_t* W8, cudaStream_t stream) {
   const int threads = 256;
-  codes_to_fp8_kernel<<<grid_for((numel >> 4) + 1, threads), threads, 0, stream>>>(W, numel, W8);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(codes_to_fp8_kernel, grid_for((numel >> 4) + 1, threads), threads, 0, stream,
+                    W, numel, W8);
 }
 
 int launch_codes_to_fp8_split(const int8_t* W, int64_t N, int64_t K, uint8_t* W8,
                               cudaStream_t stream) {
   const int threads = 256;
-  codes_to_fp8_split_kernel<<<grid_for(N * (K >> 4), threads), threads, 0, stream>>>(W, N, K, W8);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(codes_to_fp8_split_kernel, grid_for(N * (K >> 4), threads), threads, 0, stream,
+                    W, N, K, W8);
 }
 
 int launch_codes_to_bf16(const int8_t* W, int64_t numel, uint16_t* W_img, cudaStream_t stream) {
   const int threads = 256;
-  codes_to_bf16_kernel<<<grid_for((numel >> 6) + 1, threads), threads, 0, stream>>>(W, numel, W_img);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(codes_to_bf16_kernel, grid_for((numel >> 6) + 1, threads), threads, 0, stream,
+                    W, numel, W_img);
 }
 
 int launch_absmean_partial(const float* W0, int64_t numel, double* ws, cudaStream_t stream) {

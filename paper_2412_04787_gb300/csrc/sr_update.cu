@@ -88,6 +88,8 @@ __global__ void __launch_bounds__(kThreads)
                      float* __restrict__ v, int64_t numel, const UpdateConsts uc_arg,
                      const UpdateConsts* __restrict__ uc_dev, unsigned long long* changed,
                      uint16_t* __restrict__ img, uint8_t* __restrict__ img8, int64_t img8_k) {
+  dep_wait();
+  dep_trigger();
   uint8_t* Wp = reinterpret_cast<uint8_t*>(W);
   const UpdateConsts uc = DEV ? *uc_dev : uc_arg;
   const int64_t ngroups = numel >> 2;
@@ -162,6 +164,8 @@ __global__ void __launch_bounds__(kThreads)
 __global__ void __launch_bounds__(kThreads)
     slab_sum_kernel(const float* __restrict__ slabs, int nsplit, long long slab,
                     float* __restrict__ out) {
+  dep_wait();
+  dep_trigger();
   const int64_t ngroups = slab >> 2;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
   for (int64_t gi = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; gi < ngroups;
@@ -223,6 +227,8 @@ __global__ void __launch_bounds__(kThreads, 3)
                        float* __restrict__ dW_out, const UpdateConsts uc1, int split,
                        bool col_major, uint16_t* __restrict__ img_next,
                        uint8_t* __restrict__ img8_next, bool img8_split) {
+  dep_wait();
+  dep_trigger();
   const UpdateConsts uc = DEV ? *uc_dev : uc_arg;
   uint8_t* Wp = reinterpret_cast<uint8_t*>(W);
   const int64_t ngroups = static_cast<int64_t>(tail) * 16384;  // 256 x 256 / 4 per tile
@@ -333,16 +339,17 @@ int stream_blocks(int64_t numel) {
 namespace {
 
 template <bool packed, bool DEV, bool SLABS>
-void sr_launch(const float* grad, int splits, long long slab, float* g_out, int8_t* W, float* m,
-               float* v, int64_t numel, const UpdateConsts& uc, const UpdateConsts* uc_dev,
+int sr_launch(const float* grad, int splits, long long slab, float* g_out, int8_t* W, float* m,
+              float* v, int64_t numel, const UpdateConsts& uc, const UpdateConsts* uc_dev,
                unsigned long long* changed, cudaStream_t stream, uint16_t* img = nullptr,
                uint8_t* img8 = nullptr, int64_t img8_k = 0) {
-  sr_update_kernel<packed, DEV, SLABS><<<stream_blocks(numel), kThreads, 0, stream>>>(
-      grad, splits, slab, g_out, W, m, v, numel, uc, uc_dev, changed, img, img8, img8_k);
+  return launch_dep(sr_update_kernel<packed, DEV, SLABS>, stream_blocks(numel), kThreads, 0, stream,
+                    grad, splits, slab, g_out, W, m, v, numel, uc, uc_dev, changed, img, img8,
+                    img8_k);
 }
 
 template <bool packed>
-void sr_dispatch(const float* grad, int splits, long long slab, float* g_out, int8_t* W, float* m,
+int sr_dispatch(const float* grad, int splits, long long slab, float* g_out, int8_t* W, float* m,
                  float* v, int64_t numel, const UpdateConsts& uc, const UpdateConsts* uc_dev,
                  unsigned long long* changed, cudaStream_t stream, uint16_t* img = nullptr,
                  uint8_t* img8 = nullptr, int64_t img8_k = 0) {
@@ -350,19 +357,16 @@ void sr_dispatch(const float* grad, int splits, long long slab, float* g_out, in
   const bool slabs = splits > 1 || g_out || img || img8;
   if (uc_dev) {
     if (slabs)
-      sr_launch<packed, true, true>(grad, splits, slab, g_out, W, m, v, numel, uc, uc_dev, changed,
-                                    stream, img, img8, img8_k);
-    else
-      sr_launch<packed, true, false>(grad, 1, 0, nullptr, W, m, v, numel, uc, uc_dev, changed,
-                                     stream);
-  } else {
-    if (slabs)
-      sr_launch<packed, false, true>(grad, splits, slab, g_out, W, m, v, numel, uc, nullptr,
-                                     changed, stream, img, img8, img8_k);
-    else
-      sr_launch<packed, false, false>(grad, 1, 0, nullptr, W, m, v, numel, uc, nullptr, changed,
-                                      stream);
+      return sr_launch<packed, true, true>(grad, splits, slab, g_out, W, m, v, numel, uc, uc_dev,
+                                           changed, stream, img, img8, img8_k);
+    return sr_launch<packed, true, false>(grad, 1, 0, nullptr, W, m, v, numel, uc, uc_dev, changed,
+                                          stream);
   }
+  if (slabs)
+    return sr_launch<packed, false, true>(grad, splits, slab, g_out, W, m, v, numel, uc, nullptr,
+                                          changed, stream, img, img8, img8_k);
+  return sr_launch<packed, false, false>(grad, 1, 0, nullptr, W, m, v, numel, uc, nullptr, changed,
+                                         stream);
 }
 
 }  // namespace
@@ -373,11 +377,10 @@ int launch_sr_update_slabs(const float* slabs, int splits, long long slab, int8_
                            cudaStream_t stream, bool packed, uint16_t* img, uint8_t* img8,
                            int64_t img8_k) {
   if (packed)
-    sr_dispatch<true>(slabs, splits, slab, g_out, W, m, v, numel, uc, uc_dev, changed, stream);
-  else
-    sr_dispatch<false>(slabs, splits, slab, g_out, W, m, v, numel, uc, uc_dev, changed, stream,
-                       img, img8, img8_k);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+    return sr_dispatch<true>(slabs, splits, slab, g_out, W, m, v, numel, uc, uc_dev, changed,
+                             stream);
+  return sr_dispatch<false>(slabs, splits, slab, g_out, W, m, v, numel, uc, uc_dev, changed, stream,
+                            img, img8, img8_k);
 }
 
 int launch_tail_update(const float* part, int splits, int tail, int full, int num_n, int M, int N,
@@ -403,34 +406,26 @@ int launch_tail_update(const float* part, int splits, int tail, int full, int nu
   const int64_t cap = static_cast<int64_t>(sms) * o;
   const int blocks = static_cast<int>(want < cap ? want : cap);
   if (uc_dev)
-    tail_update_kernel<true><<<blocks, kThreads, 0, stream>>>(part, splits, tail, full, num_n, M, N,
-                                                              W, packed, m, v, uc, uc_dev, changed,
-                                                              dW_out, u1, uc1 ? split : 0,
-                                                              col_major, img_next, img8_next,
-                                                              img8_split);
-  else
-    tail_update_kernel<false><<<blocks, kThreads, 0, stream>>>(part, splits, tail, full, num_n, M,
-                                                               N, W, packed, m, v, uc, nullptr,
-                                                               changed, dW_out, u1,
-                                                               uc1 ? split : 0, col_major,
-                                                               img_next, img8_next, img8_split);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+    return launch_dep(tail_update_kernel<true>, blocks, kThreads, 0, stream, part, splits, tail,
+                      full, num_n, M, N, W, packed, m, v, uc, uc_dev, changed, dW_out, u1,
+                      uc1 ? split : 0, col_major, img_next, img8_next, img8_split);
+  return launch_dep(tail_update_kernel<false>, blocks, kThreads, 0, stream, part, splits, tail,
+                    full, num_n, M, N, W, packed, m, v, uc, nullptr, changed, dW_out, u1,
+                    uc1 ? split : 0, col_major, img_next, img8_next, img8_split);
 }
 
 int launch_slab_sum(const float* slabs, int splits, long long slab, float* out,
                     cudaStream_t stream) {
-  slab_sum_kernel<<<stream_blocks(slab), kThreads, 0, stream>>>(slabs, splits, slab, out);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+  return launch_dep(slab_sum_kernel, stream_blocks(slab), kThreads, 0, stream, slabs, splits, slab,
+                    out);
 }
 
 int launch_sr_update(const float* grad, int8_t* W, float* m, float* v, int64_t numel,
                      const UpdateConsts& uc, const UpdateConsts* uc_dev,
                      unsigned long long* changed, cudaStream_t stream, bool packed) {
   if (packed)
-    sr_dispatch<true>(grad, 1, 0, nullptr, W, m, v, numel, uc, uc_dev, changed, stream);
-  else
-    sr_dispatch<false>(grad, 1, 0, nullptr, W, m, v, numel, uc, uc_dev, changed, stream);
-  return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+    return sr_dispatch<true>(grad, 1, 0, nullptr, W, m, v, numel, uc, uc_dev, changed, stream);
+  return sr_dispatch<false>(grad, 1, 0, nullptr, W, m, v, numel, uc, uc_dev, changed, stream);
 }
 
 }  // namespace dqt
