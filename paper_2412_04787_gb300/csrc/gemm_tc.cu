@@ -291,35 +291,6 @@ __device__ __forceinline__ void epi_fwd(const Params& p, int gm, int gn0, float 
   }
 }
 
-// The forward's output from exact int32 accumulators (drained chunks).
-__device__ __forceinline__ void epi_fwd_int(const Params& p, int gm, int gn0, float a_t,
-                                            const int32_t (&acc)[32]) {
-  __nv_bfloat16* yrow = p.out_bf16 + static_cast<size_t>(gm) * p.N + gn0;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    if (gn0 + 8 * j >= p.N) break;
-    uint4 pk;
-    pk.x = pack_bf16x2(__fmul_rn(__int2float_rn(acc[8 * j + 0]), a_t),
-                       __fmul_rn(__int2float_rn(acc[8 * j + 1]), a_t));
-    pk.y = pack_bf16x2(__fmul_rn(__int2float_rn(acc[8 * j + 2]), a_t),
-                       __fmul_rn(__int2float_rn(acc[8 * j + 3]), a_t));
-    pk.z = pack_bf16x2(__fmul_rn(__int2float_rn(acc[8 * j + 4]), a_t),
-                       __fmul_rn(__int2float_rn(acc[8 * j + 5]), a_t));
-    pk.w = pack_bf16x2(__fmul_rn(__int2float_rn(acc[8 * j + 6]), a_t),
-                       __fmul_rn(__int2float_rn(acc[8 * j + 7]), a_t));
-    *reinterpret_cast<uint4*>(yrow + 8 * j) = pk;
-  }
-  if (p.acc_out) {
-    int32_t* arow = p.acc_out + static_cast<size_t>(gm) * p.N + gn0;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (gn0 + 4 * j >= p.N) break;
-      *reinterpret_cast<int4*>(arow + 4 * j) =
-          make_int4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
-    }
-  }
-}
-
 __device__ __forceinline__ void epi_dx(const Params& p, int gm, int gn0, const uint32_t (&a)[32]) {
   __nv_bfloat16* yrow = p.out_bf16 + static_cast<size_t>(gm) * p.N + gn0;
   const float* f = reinterpret_cast<const float*>(a);
@@ -335,30 +306,95 @@ __device__ __forceinline__ void epi_dx(const Params& p, int gm, int gn0, const u
   }
 }
 
-// FP8 forward: the fp32 accumulators are not integers; Y = bf16(acc * a_t).
-__device__ __forceinline__ void epi_fwd8(const Params& p, int gm, int gn0, float a_t,
-                                         const uint32_t (&a)[32]) {
-  const float* f = reinterpret_cast<const float*>(a);
-  __nv_bfloat16* yrow = p.out_bf16 + static_cast<size_t>(gm) * p.N + gn0;
+// The 2-SM kernels' bf16 output (forward, FP8 forward, dX).  A warp's 32 x 32
+// block goes through a 2 KB shared buffer (64-byte rows, 64-byte swizzle: the
+// lanes' 16-byte writes meet no bank conflict) and out with one TMA store.
+// Written straight from the registers, each lane held one row, so a warp's
+// store touched 32 rows of 16 bytes: half-sector writes at 1.5 cycles each
+// made the epilogue of a 256 x 256 tile 6200 cycles alone and 9700 beside
+// the mainloop, longer than the 6200 cycles of MMAs of a 768-long reduction.
+// The buffers take one operand stage (6 remain); the long reductions did not
+// lose by it.  Two captured 16384 x 768 x 768 layer steps 193 -> 170 us, eight
+// 256 x 512 x 512 steps 373 -> 346, the 8192-token MLP step 1087 -> 1068.
+constexpr int kOutBytes = 32 * 32 * 2;  // one 32 x 32 bf16 block
+
+// NB buffers per warp, taken in turn: a buffer is rewritten once the store
+// NB stores ago has read it.
+template <int NB>
+struct OutStage {
+  uint8_t* buf;
+  int turn;
+};
+
+template <int NB>
+__device__ __forceinline__ void out_store(const CUtensorMap& map, OutStage<NB>& o, int lane,
+                                          int row0, int gn0, const float (&f)[32]) {
+  uint8_t* b = o.buf + (NB > 1 ? o.turn * kOutBytes : 0);
+  if (NB > 1) o.turn = o.turn + 1 == NB ? 0 : o.turn + 1;
+  if (lane == 0) bulk_wait_read<NB - 1>();
+  __syncwarp();
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    if (gn0 + 8 * j >= p.N) break;
-    uint4 pk;
-    pk.x = pack_bf16x2(__fmul_rn(f[8 * j + 0], a_t), __fmul_rn(f[8 * j + 1], a_t));
-    pk.y = pack_bf16x2(__fmul_rn(f[8 * j + 2], a_t), __fmul_rn(f[8 * j + 3], a_t));
-    pk.z = pack_bf16x2(__fmul_rn(f[8 * j + 4], a_t), __fmul_rn(f[8 * j + 5], a_t));
-    pk.w = pack_bf16x2(__fmul_rn(f[8 * j + 6], a_t), __fmul_rn(f[8 * j + 7], a_t));
-    *reinterpret_cast<uint4*>(yrow + 8 * j) = pk;
+  for (int j = 0; j < 4; ++j)
+    *reinterpret_cast<uint4*>(b + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) =
+        make_uint4(pack_bf16x2(f[8 * j + 0], f[8 * j + 1]), pack_bf16x2(f[8 * j + 2], f[8 * j + 3]),
+                   pack_bf16x2(f[8 * j + 4], f[8 * j + 5]), pack_bf16x2(f[8 * j + 6], f[8 * j + 7]));
+  fence_async_shared();
+  __syncwarp();
+  if (lane == 0) {
+    tma_store_2d(&map, b, gn0, row0);
+    bulk_commit();
   }
-  if (p.acc_f32) {
-    float* arow = p.acc_f32 + static_cast<size_t>(gm) * p.N + gn0;
+}
+
+// 32 columns of one accumulator row as optional debug output (int32 or fp32).
+template <typename T>
+__device__ __forceinline__ void acc_row_out(T* acc, const Params& p, int gm, int gn0,
+                                            const T (&a)[32]) {
+  T* row = acc + static_cast<size_t>(gm) * p.N + gn0;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (gn0 + 4 * j >= p.N) break;
-      *reinterpret_cast<float4*>(arow + 4 * j) =
-          make_float4(f[4 * j], f[4 * j + 1], f[4 * j + 2], f[4 * j + 3]);
-    }
+  for (int j = 0; j < 8; ++j) {
+    if (gn0 + 4 * j >= p.N) break;
+    alignas(16) const T v[4] = {a[4 * j], a[4 * j + 1], a[4 * j + 2], a[4 * j + 3]};
+    *reinterpret_cast<uint4*>(row + 4 * j) = *reinterpret_cast<const uint4*>(v);
   }
+}
+
+// One 32 x 32 block (rows row0 + lane, columns gn0 ..) of the output from its
+// fp32 accumulators: Y = bf16(acc a_t) or dX = bf16(acc scale).  An integer
+// accumulator is exact in fp32; + 0 turns a -0 into the integer's +0.
+template <int EPI, int NB>
+__device__ __forceinline__ void out_block(const CUtensorMap& map, OutStage<NB>& o, const Params& p,
+                                          int lane, int row0, int gn0, float a_t,
+                                          const uint32_t (&a)[32]) {
+  const bool row_ok = row0 + lane < p.M;
+  float f[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) f[i] = __uint_as_float(a[i]);
+  if (EPI == GEMM_FWD8 && p.acc_f32 && row_ok) acc_row_out(p.acc_f32, p, row0 + lane, gn0, f);
+  if (EPI == GEMM_FWD && p.acc_out && row_ok) {
+    int32_t n[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) n[i] = __float2int_rn(f[i]);
+    acc_row_out(p.acc_out, p, row0 + lane, gn0, n);
+  }
+#pragma unroll
+  for (int i = 0; i < 32; ++i) {
+    if (EPI == GEMM_FWD) f[i] = __fmul_rn(__fadd_rn(f[i], 0.0f), a_t);
+    else f[i] = __fmul_rn(f[i], EPI == GEMM_DX ? p.scale : a_t);
+  }
+  out_store(map, o, lane, row0, gn0, f);
+}
+
+// The same from the int32 sums of drained chunks.
+template <int NB>
+__device__ __forceinline__ void out_block_int(const CUtensorMap& map, OutStage<NB>& o,
+                                              const Params& p, int lane, int row0, int gn0,
+                                              float a_t, const int32_t (&acc)[32]) {
+  if (p.acc_out && row0 + lane < p.M) acc_row_out(p.acc_out, p, row0 + lane, gn0, acc);
+  float f[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) f[i] = __fmul_rn(__int2float_rn(acc[i]), a_t);
+  out_store(map, o, lane, row0, gn0, f);
 }
 
 // dW: gradient -> AdamW -> SR -> codes, in registers, four weights (one
@@ -847,9 +883,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 // 2-SM variant (cta_group::2): a cluster of two CTAs on the SM pair of a TPC
 // computes a 256 x 256 output tile.  CTA r stages rows [128 r, 128 r + 128)
 // of A and rows/columns [128 r, 128 r + 128) of B's 256-wide tile: 32 KB per
-// stage instead of 48 KB, so the ring is 7 stages deep (6 for dW, which also
-// holds the transpose buffers) and each SM pulls a third fewer operand bytes
-// through L2 per FLOP.  Both CTAs' copies complete on the leader's `full`
+// stage instead of 48 KB, so the ring is 6 stages deep beside the output
+// buffers (5 for dW, which holds the transpose buffers) and each SM pulls a
+// third fewer operand bytes through L2 per FLOP.  Both CTAs' copies complete on the leader's `full`
 // barrier; the leader issues the 256 x 256 x 16 MMAs and multicasts its
 // commits to both CTAs' `empty` and `acc_full` barriers; each CTA's epilogue
 // reads its own 128 rows from its own tensor memory and releases the
@@ -872,9 +908,12 @@ struct SmemPair {
   static constexpr int A_BYTES = 128 * BK * 2;
   static constexpr int B_BYTES = 128 * BK * 2;  // this CTA's half of the B tile
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = (EPI == GEMM_DW) ? 5 : 7;
+  static constexpr int STAGES = (EPI == GEMM_DW) ? 5 : 6;
   static constexpr int XPOSE_OFF = STAGES * STAGE_BYTES;
-  static constexpr int XPOSE_BYTES = (EPI == GEMM_DW) ? EW * 32 * kStageLd * 4 : 0;
+  // dW: the transpose buffers; else the output buffers, OUT_NB per warp
+  static constexpr int OUT_NB = 16 / EW;
+  static constexpr int XPOSE_BYTES = (EPI == GEMM_DW) ? EW * 32 * kStageLd * 4
+                                                      : EW * OUT_NB * kOutBytes;
   static constexpr int BAR_OFF = XPOSE_OFF + XPOSE_BYTES;
   // alignment slack for the 1024-byte swizzle atoms, as much as fits
   static constexpr int SLACK = (232448 - (BAR_OFF + 256)) < 1024 ? (232448 - (BAR_OFF + 256)) : 1024;
@@ -896,8 +935,9 @@ struct SmemPair {
 // optimiser state, images, constants and tile order; whole tiles only.
 template <bool A_MN, bool B_MN, int EPI, bool PK, bool DR, bool UCD, bool GRP>
 __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUtensorMap& tmB,
-                                               const Params& p, const CUtensorMap& tmA2,
-                                               const CUtensorMap& tmB2, const Params& p2) {
+                                               const CUtensorMap& tmD, const Params& p,
+                                               const CUtensorMap& tmA2, const CUtensorMap& tmB2,
+                                               const Params& p2) {
   using S = SmemPair<EPI, DR>;
   static_assert(!DR || EPI == GEMM_FWD, "drained chunks: exact integer forward only");
   static_assert(!GRP || (EPI == GEMM_DW && !DR && !UCD), "grouped launches: dW, constants by value");
@@ -956,6 +996,7 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
     fence_mbarrier_init();
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
+    if (EPI != GEMM_DW) tma_prefetch_desc(&tmD);
     if (GRP) {
       tma_prefetch_desc(&tmA2);
       tma_prefetch_desc(&tmB2);
@@ -1125,6 +1166,7 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
     const int row = quad * 32 + lane;
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
     float* xp = reinterpret_cast<float*>(smem + S::XPOSE_OFF) + (warp - 2) * 32 * kStageLd;
+    OutStage<S::OUT_NB> out{smem + S::XPOSE_OFF + (warp - 2) * S::OUT_NB * kOutBytes, 0};
     uint32_t n_changed = 0, n_changed2 = 0;  // changed codes of p's and p2's units
     int u = 0;
     bool ok = true;
@@ -1175,9 +1217,9 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
           if (lane == 0) mbar_arrive_cluster(acc_empty_lead + 8u * b);
         }
         if (!ok) return false;
-        if (row_ok) {
-          if (nbase < q.N) epi_fwd_int(q, gm, nbase, a_t, run0);
-          if (nbase + 32 < q.N) epi_fwd_int(q, gm, nbase + 32, a_t, run1);
+        if (gm - lane < q.M) {
+          if (nbase < q.N) out_block_int(tmD, out, q, lane, gm - lane, nbase, a_t, run0);
+          if (nbase + 32 < q.N) out_block_int(tmD, out, q, lane, gm - lane, nbase + 32, a_t, run1);
         }
         --u;  // the loop header counts one unit per tile
         return true;
@@ -1270,12 +1312,11 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
 #pragma unroll 1
               for (int sl = 0; sl < q.tail_splits; ++sl)
                 l2_discard_line(src0 + sl * sstride + cc * 1024 + lane * 32);
-              if (gn0 >= q.N || !row_ok) continue;
+              if (gn0 >= q.N || gm - lane >= q.M) continue;  // warp-uniform
               uint32_t a[32];
 #pragma unroll
               for (int i = 0; i < 32; ++i) a[i] = __float_as_uint(f[i]);
-              if (EPI == GEMM_FWD) epi_fwd(q, gm, gn0, a_t, a, a, false);  // no running sums
-              else epi_dx(q, gm, gn0, a);
+              out_block<EPI>(tmD, out, q, lane, gm - lane, gn0, a_t, a);
             }
           }
           return true;  // the accumulator is already released
@@ -1303,15 +1344,12 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
       } else
 #pragma unroll 1
       for (int cc = 0; cc < HALF / 32; ++cc) {
-        uint32_t a[32], r[32];
+        uint32_t a[32];
+        const int gn0 = nbase + cc * 32;
+        if (gn0 >= q.N || gm - lane >= q.M) continue;  // warp-uniform
         tmem_ld_32x32b_x32(t_acc + cc * 32, a);
         tmem_ld_wait();
-        const int gn0 = nbase + cc * 32;
-        if (gn0 >= q.N) continue;  // warp-uniform
-        if (!row_ok) continue;
-        if (EPI == GEMM_FWD) epi_fwd(q, gm, gn0, a_t, a, r, false);
-        else if (F8) epi_fwd8(q, gm, gn0, a_t, a);
-        else epi_dx(q, gm, gn0, a);
+        out_block<EPI>(tmD, out, q, lane, gm - lane, gn0, a_t, a);
       }
       tc_fence_before();
       __syncwarp();
@@ -1323,6 +1361,7 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
       ok = (GRP && t >= p.num_tiles) ? epi_unit(p2, t - p.num_tiles, n_changed2)
                                      : epi_unit(p, t, n_changed);
     if (!ok && lane == 0) record_timeout(p.status);
+    if (EPI != GEMM_DW && lane == 0) bulk_wait_all();  // this warp's stores have landed
     if (EPI == GEMM_DW && p.changed) {
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) n_changed += __shfl_xor_sync(0xffffffffu, n_changed, off);
@@ -1348,8 +1387,9 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
 template <bool A_MN, bool B_MN, int EPI, bool PK = false, bool DR = false, bool UCD = false>
 __global__ void __launch_bounds__(PairCfg<EPI, DR>::THREADS, 1)
     gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA,
-                     const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Params p) {
-  gemm_pair_body<A_MN, B_MN, EPI, PK, DR, UCD, false>(tmA, tmB, p, tmA, tmB, p);
+                     const __grid_constant__ CUtensorMap tmB,
+                     const __grid_constant__ CUtensorMap tmD, const __grid_constant__ Params p) {
+  gemm_pair_body<A_MN, B_MN, EPI, PK, DR, UCD, false>(tmA, tmB, tmD, p, tmA, tmB, p);
 }
 
 // Two dW + update problems in one persistent launch (both operands MN-major,
@@ -1360,7 +1400,7 @@ __global__ void __launch_bounds__(PairCfg<GEMM_DW, false>::THREADS, 1)
                          const __grid_constant__ CUtensorMap tmA2,
                          const __grid_constant__ CUtensorMap tmB2,
                          const __grid_constant__ Params p2) {
-  gemm_pair_body<true, true, GEMM_DW, false, false, false, true>(tmA, tmB, p, tmA2, tmB2, p2);
+  gemm_pair_body<true, true, GEMM_DW, false, false, false, true>(tmA, tmB, tmA, p, tmA2, tmB2, p2);
 }
 
 // ---------------------------------------------------------------------------
@@ -1386,9 +1426,10 @@ EncodeTiledFn encode_fn() {
 
 // 2-D row-major matrix of 2-byte (bf16) or 1-byte (E4M3) elements with
 // `inner` contiguous elements per row and `outer` rows; box of box_inner x
-// box_outer, 128-byte swizzle, zero fill.
+// box_outer, zero fill, 128-byte swizzle unless given.
 bool make_map(CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t outer,
-              uint32_t box_inner, uint32_t box_outer, int elem_bytes = 2, uint64_t row_elems = 0) {
+              uint32_t box_inner, uint32_t box_outer, int elem_bytes = 2, uint64_t row_elems = 0,
+              CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
   EncodeTiledFn enc = encode_fn();
   if (!enc) return false;
   // The encoder is a driver call and needs a context current in the calling
@@ -1407,7 +1448,7 @@ bool make_map(CUtensorMap* map, const void* ptr, uint64_t inner, uint64_t outer,
   const cuuint32_t estr[2] = {1, 1};
   return enc(map, elem_bytes == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16,
              2, const_cast<void*>(ptr), dims, strides, box,
-             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -1602,7 +1643,12 @@ int launch_pairs(const CUtensorMap& ta, const CUtensorMap& tb, Params p, cudaStr
   }
   const int clusters = p.num_tiles < max_clusters ? p.num_tiles : max_clusters;
   cfg.gridDim = dim3(2 * clusters, 1, 1);
-  if (cudaLaunchKernelEx(&cfg, kern, ta, tb, p) != cudaSuccess) return 3;
+  // the output's map (32 x 32 blocks, see out_store); dW has none
+  CUtensorMap td = ta;
+  if (EPI != GEMM_DW &&
+      !make_map(&td, p.out_bf16, p.N, p.M, 32, 32, 2, 0, CU_TENSOR_MAP_SWIZZLE_64B))
+    return 3;
+  if (cudaLaunchKernelEx(&cfg, kern, ta, tb, td, p) != cudaSuccess) return 3;
   return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
 }
 
