@@ -321,9 +321,10 @@ int dqt_bitlinear_bwd_dw_update_img(const dqt_bf16* dY, const dqt_bf16* Xdq, int
 /* Workspace (bytes, 16-byte aligned device memory) that lets
  * dqt_bitlinear_bwd_dw_update_img (and the rest of dqt_bitlinear_bwd_dw_update's
  * workspace) cut token reductions into slices:
- *  - a weight gradient whose output is too small to occupy the GPU (few
- *    256 x 256 tiles, long token reduction) is reduced in token slices
- *    throughout;
+ *  - a weight gradient whose output is too small to occupy the GPU (at most
+ *    3/4 as many 256 x 256 tiles as SM pairs) is reduced in token slices
+ *    throughout (one, when the tiles or the reduction allow no more: the
+ *    fused kernel's update of so few tiles would use only their SMs);
  *  - otherwise, when the output's tiles do not fill the last wave of SM pairs,
  *    the tiles of that wave are reduced in token slices, so that the last
  *    wave is short.

@@ -561,7 +561,7 @@ size_t dqt_bwd_dw_img_workspace_size(int64_t T, int64_t N, int64_t K) {
   if (T <= 0 || N <= 0 || K <= 0 || T > kMaxDim || N > kMaxDim || K > kMaxDim) return 0;
   if (dqt::gemm_mode() != 0) return 0;
   const int s = dqt::dw_splits(static_cast<int>(N), static_cast<int>(K), static_cast<int>(T));
-  if (s > 1) return static_cast<size_t>(s) * static_cast<size_t>(N) * static_cast<size_t>(K) * 4u;
+  if (s > 0) return static_cast<size_t>(s) * static_cast<size_t>(N) * static_cast<size_t>(K) * 4u;
   // last-wave tail: at most one 256 x 256 fp32 slice partial per cluster (at
   // most one cluster per SM pair on any launch)
   int dev = 0, sms = 148;

@@ -99,8 +99,9 @@ struct GemmLaunch {
   int a_wrap;
 };
 
-// Token slices the 2-SM dW GEMM of an M x N output reduced over Kred uses
-// when given a workspace of dw_splits * M * N floats (1 = no split).
+// Token slices the 2-SM dW GEMM of an M x N output reduced over Kred writes
+// when given a workspace of dw_splits * M * N floats, their sum and the update
+// then a streaming pass (0 = the fused kernel).
 int dw_splits(int M, int N, int Kred);
 
 // The last-wave tail of a 2-SM dW GEMM on `clusters` clusters: `tail` tiles

@@ -19,15 +19,23 @@ constexpr int kThreads = 256;
 // The gradient of element e is grad[e], or, with nsplit > 1 partial slabs of
 // `slab` elements each (a split-T weight gradient), their sum taken in slab
 // order; g_out (optional) receives that gradient.
+// The slabs are read four at a time, so that their loads are in flight together.
 __device__ __forceinline__ float4 slab_grad4(const float* __restrict__ grad, int nsplit,
                                              long long slab, int64_t e) {
   float4 g4 = __ldcs(reinterpret_cast<const float4*>(grad + e));
-  for (int s = 1; s < nsplit; ++s) {
-    const float4 h = __ldcs(reinterpret_cast<const float4*>(grad + s * slab + e));
-    g4.x = __fadd_rn(g4.x, h.x);
-    g4.y = __fadd_rn(g4.y, h.y);
-    g4.z = __fadd_rn(g4.z, h.z);
-    g4.w = __fadd_rn(g4.w, h.w);
+  for (int s = 1; s < nsplit; s += 4) {
+    float4 h[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (s + j < nsplit) h[j] = __ldcs(reinterpret_cast<const float4*>(grad + (s + j) * slab + e));
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (s + j < nsplit) {
+        g4.x = __fadd_rn(g4.x, h[j].x);
+        g4.y = __fadd_rn(g4.y, h[j].y);
+        g4.z = __fadd_rn(g4.z, h[j].z);
+        g4.w = __fadd_rn(g4.w, h[j].w);
+      }
   }
   return g4;
 }
@@ -82,7 +90,7 @@ __device__ __forceinline__ void store_images4(uint16_t* img, uint8_t* img8, int6
 // img8 E4M3, direct or split as in store_e4m3_4; int8 codes only) written
 // beside them.  The plain instance is the leanest stream.
 template <bool packed, bool DEV, bool SLABS>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, SLABS ? 4 : 1)
     sr_update_kernel(const float* __restrict__ grad, int nsplit, long long slab,
                      float* __restrict__ g_out, int8_t* __restrict__ W, float* __restrict__ m,
                      float* __restrict__ v, int64_t numel, const UpdateConsts uc_arg,
@@ -98,12 +106,12 @@ __global__ void __launch_bounds__(kThreads)
   for (int64_t gi = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; gi < ngroups;
        gi += stride) {
     const int64_t e = gi << 2;
-    const float4 g4 = SLABS ? slab_grad4(grad, nsplit, slab, e)
-                            : __ldcs(reinterpret_cast<const float4*>(grad + e));
-    if (SLABS && g_out) __stcs(reinterpret_cast<float4*>(g_out + e), g4);
     float4 m4 = __ldcs(reinterpret_cast<const float4*>(m + e));
     float4 v4 = __ldcs(reinterpret_cast<const float4*>(v + e));
     const char4 c4 = packed ? tern_unpack4(Wp[gi]) : *reinterpret_cast<const char4*>(W + e);
+    const float4 g4 = SLABS ? slab_grad4(grad, nsplit, slab, e)
+                            : __ldcs(reinterpret_cast<const float4*>(grad + e));
+    if (SLABS && g_out) __stcs(reinterpret_cast<float4*>(g_out + e), g4);
     uint4 w = make_uint4(0, 0, 0, 0);
     if (uc.round_mode == 0)
       w = sr_words(global_blk(uc, static_cast<uint64_t>(gi)), uc.step_lo, uc.tensor_id, uc.key0,
