@@ -90,7 +90,7 @@ __device__ __forceinline__ void store_images4(uint16_t* img, uint8_t* img8, int6
 // img8 E4M3, direct or split as in store_e4m3_4; int8 codes only) written
 // beside them.  The plain instance is the leanest stream.
 template <bool packed, bool DEV, bool SLABS>
-__global__ void __launch_bounds__(kThreads, SLABS ? 4 : 1)
+__global__ void __launch_bounds__(kThreads, SLABS ? 4 : 5)
     sr_update_kernel(const float* __restrict__ grad, int nsplit, long long slab,
                      float* __restrict__ g_out, int8_t* __restrict__ W, float* __restrict__ m,
                      float* __restrict__ v, int64_t numel, const UpdateConsts uc_arg,
