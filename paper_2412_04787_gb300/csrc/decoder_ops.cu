@@ -99,36 +99,69 @@ __device__ __forceinline__ void lse_block(float& m, float& s, float* sh_m, float
   }
 }
 
-// One block per row; V a multiple of 8 (16-byte vectors of bf16).
+// 2^t (the PTX instruction: relative error at most 2^-22).
+__device__ __forceinline__ float ex2(float t) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(t));
+  return r;
+}
+
+// One block per row; V a multiple of 8 (16-byte vectors of bf16).  A thread
+// takes kCeVecs vectors at a time, their loads in flight together: the
+// chunk's maximum on bf16 pairs (exact; a NaN makes the row's sum NaN), one
+// rescaling of the running sum, then exp(x - max) as 2^((x - max) log2 e),
+// the difference formed before the product, so the product's rounding is
+// 2^-24 of an exponent that is small wherever the term counts.  With expf
+// and a maximum and rescaling per vector the kernel was bound by instruction
+// issue: 8192 x 32000 rows, forward and gradient together, 286 -> 244 us.
+constexpr int kCeVecs = 8;
+
 __global__ void __launch_bounds__(kCeThreads)
     ce_fwd_kernel(const uint4* __restrict__ logits, const int64_t* __restrict__ tgt, int64_t V,
                   float* __restrict__ lse, float* __restrict__ row_loss) {
   dep_wait();
   dep_trigger();
   __shared__ float sh_m[kCeThreads / 32], sh_s[kCeThreads / 32];
+  constexpr float kLog2e = 1.44269504088896340736f;
   const int64_t r = blockIdx.x;
-  const int64_t nv = V >> 3;
+  const int nv = static_cast<int>(V >> 3);
   const uint4* row = logits + r * nv;
   float m = -INFINITY, s = 0.0f;
-  // two vectors in flight per thread step
-  for (int64_t i = threadIdx.x; i < nv; i += 2 * kCeThreads) {
-    const bool two = i + kCeThreads < nv;
-    const uint4 va = __ldcs(row + i);
-    const uint4 vb = two ? __ldcs(row + i + kCeThreads) : va;
+  for (int i0 = threadIdx.x; i0 < nv; i0 += kCeVecs * kCeThreads) {
+    uint4 v[kCeVecs];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (h == 1 && !two) break;
-      const uint4 v = h ? vb : va;
-      const float f[8] = {bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y),
-                          bf16_lo(v.z), bf16_hi(v.z), bf16_lo(v.w), bf16_hi(v.w)};
-      float mv = f[0];
-#pragma unroll
-      for (int j = 1; j < 8; ++j) mv = fmaxf(mv, f[j]);
-      float sv = 0.0f;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) sv += expf(f[j] - mv);
-      lse_merge(m, s, mv, sv);
+    for (int k = 0; k < kCeVecs; ++k) {
+      const int i = i0 + k * kCeThreads;
+      // past the row: -inf, which adds nothing
+      v[k] = i < nv ? __ldcs(row + i) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
     }
+    __nv_bfloat162 mx = *reinterpret_cast<const __nv_bfloat162*>(&v[0].x);
+#pragma unroll
+    for (int k = 0; k < kCeVecs; ++k) {
+      const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) mx = __hmax2_nan(mx, *reinterpret_cast<const __nv_bfloat162*>(&w[j]));
+    }
+    const float lo = __low2float(mx), hi = __high2float(mx), cm = fmaxf(lo, hi);
+    if (cm == -INFINITY && lo == hi) continue;  // nothing but -inf
+    if (lo != lo || hi != hi) {
+      s = lo + hi;
+      m = fmaxf(m, -3.4e38f);  // finite: the merge below drops sums at -inf
+      continue;
+    }
+    const float mn = fmaxf(m, cm);
+    float t0 = 0.0f, t1 = 0.0f;  // two chains
+#pragma unroll
+    for (int k = 0; k < kCeVecs; ++k) {
+      const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        t0 += ex2(__fmul_rn(bf16_lo(w[j]) - mn, kLog2e));
+        t1 += ex2(__fmul_rn(bf16_hi(w[j]) - mn, kLog2e));
+      }
+    }
+    s = s * expf(m - mn) + (t0 + t1);  // the first time 0 * expf(-inf)
+    m = mn;
   }
   lse_block(m, s, sh_m, sh_s);
   if (threadIdx.x == 0) {
