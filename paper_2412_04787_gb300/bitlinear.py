@@ -48,24 +48,26 @@ class _QuantCache:
     ref = None
     version = -1
     act = None
+    xdq = False
     result = None
 
 
-def _quantised(x, x2, act):
+# want_xdq: the dequantised image too, which only a backward reads
+def _quantised(x, x2, act, want_xdq):
     c = _QuantCache
     try:
         version = x._version
     except RuntimeError:  # inference tensors keep no version counter: no sharing
         version = None
     if (version is not None and c.ref is not None and c.ref() is x and c.version == version
-            and c.act == act):
+            and c.act == act and (c.xdq or not want_xdq)):
         return c.result
     if act == "fp8":
-        res = dqt.dqt_act_quant_fp8(x2)
+        res = dqt.dqt_act_quant_fp8(x2, want_xdq=want_xdq)
     else:
-        res = dqt.dqt_act_quant_images(x2, want=("Xq_img", "Xdq"))
+        res = dqt.dqt_act_quant_images(x2, want=("Xq_img", "Xdq") if want_xdq else ("Xq_img",))
     if version is not None:
-        c.ref, c.version, c.act, c.result = weakref.ref(x), version, act, res
+        c.ref, c.version, c.act, c.xdq, c.result = weakref.ref(x), version, act, want_xdq, res
     else:
         c.ref, c.result = None, None
     return res
@@ -73,19 +75,19 @@ def _quantised(x, x2, act):
 
 class _BitLinearFn(torch.autograd.Function):
     @staticmethod
-    def forward(ctx, x, anchor, layer):
+    def forward(ctx, x, anchor, layer, grad):
         K, N = layer.in_features, layer.out_features
         x2 = x.reshape(-1, K)
         if x2.dtype != torch.bfloat16:
             x2 = x2.to(torch.bfloat16)
         x2 = x2.contiguous()
         if layer.act == "fp8":
-            q8, s_x, xdq = _quantised(x, x2, "fp8")
+            q8, s_x, xdq = _quantised(x, x2, "fp8", grad)
             y = dqt.dqt_bitlinear_fwd_fp8(q8, s_x, layer.image_fp8(), float(layer.s_w),
                                           layer.grid_tuple)
             w_img = None  # dX needs the bf16 image: taken in backward
         else:
-            _, s_x, q_img, xdq = _quantised(x, x2, "int8")
+            _, s_x, q_img, xdq = _quantised(x, x2, "int8", grad)
             # the weight's code image serves the forward and, kept until the
             # backward, dX (the codes change only after dX, in the update)
             w_img = layer.image_bf16()
@@ -111,7 +113,7 @@ class _BitLinearFn(torch.autograd.Function):
         dx = dqt.dqt_bitlinear_bwd_dx_img(dy2, w_img, float(layer.s_w))
         if layer.update_in_backward:
             layer._dqt_update(dy2, xdq)
-        return dx.reshape(ctx.in_shape).to(ctx.in_dtype), None, None
+        return dx.reshape(ctx.in_shape).to(ctx.in_dtype), None, None, None
 
 
 class DQTBitLinear(torch.nn.Module):
@@ -207,7 +209,8 @@ class DQTBitLinear(torch.nn.Module):
         self.tensor_id = int(state["tensor_id"])
 
     def forward(self, x):
-        return _BitLinearFn.apply(x, self._anchor, self)
+        # (inside the function gradients are always off)
+        return _BitLinearFn.apply(x, self._anchor, self, torch.is_grad_enabled())
 
     def int8_codes(self):
         """The codes as an int8 [N, K] tensor (unpacked if stored packed)."""

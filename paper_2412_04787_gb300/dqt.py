@@ -209,10 +209,14 @@ def _check(rc, where):
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _need(t, name, dtype, shape=None):
+    # torch.Size is a tuple: it compares with the callers' tuples as it is
+    if (t is not None and t.is_cuda and t.dtype == dtype and t.is_contiguous()
+            and (shape is None or t.shape == shape)):
+        return t
     if t is None:
         raise ValueError("%s is required" % name)
     if not t.is_cuda:
@@ -231,8 +235,12 @@ def _opt(t, name, dtype, shape):
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    # the raw handle of torch.cuda.current_stream() without the Stream object,
+    # whose construction was a third of a call's host time (about 10 us)
+    torch.cuda._lazy_init()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def grid(bits):
