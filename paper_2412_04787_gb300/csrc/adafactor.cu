@@ -3,18 +3,19 @@
 // ICML 2018).  The second moment of an N x K gradient G is kept factored as
 // its row means R [N] and column means C [K]; there is no first moment and no
 // per-weight optimiser state, so a step reads G and the codes and writes the
-// codes.  Four passes, each HBM-bound or tiny:
+// codes.  Four launches, each HBM-bound or tiny:
 //
 //   af_sq_partials  one read of G (and the codes): per 128-column chunk row
 //                   sums and per 32-row slab column sums of g^2 + eps1, and the
 //                   sum of c^2 (for the parameter RMS), in a fixed order
-//   af_moments      R <- b2 R + (1 - b2) mean_k, C <- b2 C + (1 - b2) mean_n
-//   af_factors      one block: Rbar = mean R, and the inverse square root of
-//                   the rank-one estimate R C / Rbar as a row factor
-//                   a[n] = 1 / sqrt(R[n] / Rbar) times a column factor
-//                   b[k] = 1 / sqrt(C[k])
-//   af_usq_partials second read of G: sum of u^2, u = (g a[n]) b[k], per block
-//   af_finalize     one block: RMS(u), RMS(W) = sqrt(sum c^2 / NK) / s_w,
+//   af_moments      R <- b2 R + (1 - b2) mean_k, C <- b2 C + (1 - b2) mean_n,
+//                   and (the last row block to finish) Rbar = mean R
+//   af_usq          the inverse square root of the rank-one estimate R C / Rbar
+//                   as a row factor a[n] = 1 / sqrt(R[n] /
+//                   Rbar) times a column factor b[k] = 1 / sqrt(C[k]) (each
+//                   block forms those of its rows and columns); second read of
+//                   G: sum of u^2, u = (g a[n]) b[k], per block; the last block
+//                   to finish: RMS(u), RMS(W) = sqrt(sum c^2 / NK) / s_w,
 //                   alpha, the clipped code-domain step and the weight decay
 //   af_apply        third read of G: u = (g a[n]) b[k], x = c decay - step u,
 //                   then SR (Eq. 1) and the clamp (Eq. 5): two multiplies per
@@ -59,7 +60,8 @@ constexpr int kUnroll = 4;
 __global__ void __launch_bounds__(kThreads, 4)
     af_sq_partials_kernel(const float* __restrict__ G, const int8_t* __restrict__ W, bool packed,
                           bool need_csq, int N, int K, float eps1, float* __restrict__ rowpart,
-                          float* __restrict__ colpart, unsigned long long* __restrict__ cpart) {
+                          float* __restrict__ colpart, unsigned long long* __restrict__ cpart,
+                          unsigned int* __restrict__ done) {
   dep_wait();
   dep_trigger();
   __shared__ unsigned long long sh[kThreads / 32];
@@ -67,6 +69,8 @@ __global__ void __launch_bounds__(kThreads, 4)
   const int k0 = blockIdx.x * kColsPerBlock + threadIdx.x * 4;
   const int n0 = blockIdx.y * kRowsPerSlab;
   const bool col_ok = k0 < K;  // K is a multiple of 4: the whole float4 is in range
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2)
+    done[threadIdx.x] = 0;  // the counts of finished blocks of the two kernels that follow
   float cs[4] = {0.f, 0.f, 0.f, 0.f};
   uint32_t csq = 0;  // at most 32 rows x 4 codes x 128^2 per thread
   const int chunk = blockIdx.x * (kColsPerBlock / 128) + warp;  // this warp's 128-column chunk
@@ -127,16 +131,38 @@ __global__ void __launch_bounds__(kThreads, 4)
 __global__ void __launch_bounds__(kThreads)
     af_moments_kernel(const float* __restrict__ rowpart, const float* __restrict__ colpart,
                       int nchunks, int nslabs, int N, int K, int row_blocks, float b2, float omb2,
-                      float* __restrict__ R, float* __restrict__ C) {
+                      float* __restrict__ R, float* __restrict__ C, double* __restrict__ rsum,
+                      unsigned int* __restrict__ done, float* __restrict__ out) {
   dep_wait();
   dep_trigger();
   if (static_cast<int>(blockIdx.x) < row_blocks) {
+    __shared__ double shd[kThreads / 32];
+    __shared__ bool last_s;
     const int t = blockIdx.x * kThreads + threadIdx.x;
-    if (t >= N) return;
-    float s = 0.f;
-    for (int j = 0; j < nchunks; ++j) s += rowpart[static_cast<int64_t>(j) * N + t];
-    const float mean = __fdiv_rn(s, static_cast<float>(K));
-    R[t] = __fadd_rn(__fmul_rn(b2, R[t]), __fmul_rn(omb2, mean));
+    double rn = 0.0;
+    if (t < N) {
+      float s = 0.f;
+#pragma unroll 8
+      for (int j = 0; j < nchunks; ++j) s += rowpart[static_cast<int64_t>(j) * N + t];
+      const float mean = __fdiv_rn(s, static_cast<float>(K));
+      const float r = __fadd_rn(__fmul_rn(b2, R[t]), __fmul_rn(omb2, mean));
+      R[t] = r;
+      rn = static_cast<double>(r);
+    }
+    rn = block_sum(rn, shd);
+    if (threadIdx.x == 0) {
+      rsum[blockIdx.x] = rn;
+      __threadfence();
+      last_s = atomicAdd(done, 1u) == static_cast<unsigned int>(row_blocks) - 1u;
+      __threadfence();
+    }
+    __syncthreads();
+    if (!last_s) return;
+    // Rbar: the row blocks' fp64 sums added in order, rounded once to fp32
+    double rs = 0.0;
+    for (int i = threadIdx.x; i < row_blocks; i += kThreads) rs += __ldcg(rsum + i);
+    rs = block_sum(rs, shd);
+    if (threadIdx.x == 0) out[0] = static_cast<float>(rs / static_cast<double>(N));
     return;
   }
   __shared__ float part[8][33];
@@ -162,102 +188,97 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// Rbar (fixed-order fp64 sum of R, rounded once to fp32; every block forms
-// the same sum), then this block's slice of the factors a[n] = 1 / sqrt(R[n] /
-// Rbar) and b[k] = 1 / sqrt(C[k]) over the concatenated index n, then N + k,
-// each from correctly rounded fp32 operations.
-__global__ void __launch_bounds__(kThreads)
-    af_factors_kernel(const float* __restrict__ R, const float* __restrict__ C, int N, int K,
-                      float* __restrict__ a, float* __restrict__ b, float* __restrict__ scal) {
-  dep_wait();
-  dep_trigger();
-  __shared__ double shd[kThreads / 32];
-  __shared__ float rbar_s;
-  double rs = 0.0;
-  for (int i = threadIdx.x; i < N; i += kThreads) rs += static_cast<double>(R[i]);
-  rs = block_sum(rs, shd);
-  if (threadIdx.x == 0) {
-    rbar_s = static_cast<float>(rs / static_cast<double>(N));
-    if (blockIdx.x == 0) scal[0] = rbar_s;
-  }
-  __syncthreads();
-  const float rbar = rbar_s;
-  const int i = blockIdx.x * kThreads + threadIdx.x;
-  if (i < N)
-    a[i] = __fdiv_rn(1.0f, __fsqrt_rn(__fdiv_rn(R[i], rbar)));
-  else if (i < N + K)
-    b[i - N] = __fdiv_rn(1.0f, __fsqrt_rn(C[i - N]));
-}
-
 __device__ __forceinline__ float af_u(float g, float an, float bk) {
   return __fmul_rn(__fmul_rn(g, an), bk);
 }
 
+// The factors a[n] = 1 / sqrt(R[n] / Rbar) and b[k] = 1 / sqrt(C[k]) of this
+// block's rows and columns, each from correctly rounded fp32 operations (the
+// first block of a row or column range writes them out), and the block's sum
+// of u^2.  The block that finishes last (counted in `done`) adds the partials
+// in order and writes the step's scalars: out = {Rbar (already there), step,
+// decay, rms_u, rms_x, alpha}.  Factors and scalars had launches of their own,
+// 6.7 and 6.9 us of latency for a few thousand values (the statistics of 5632 x
+// 2048, replayed: 40.2 -> 38.0 us).
+struct FinalArgs {
+  float s_w, rho, eps2, clip_d, weight_decay;
+  int scale_parameter;
+};
+
 __global__ void __launch_bounds__(kThreads)
-    af_usq_partials_kernel(const float* __restrict__ G, const float* __restrict__ a,
-                           const float* __restrict__ b, int N, int K, float* __restrict__ upart) {
+    af_usq_kernel(const float* __restrict__ G, const float* __restrict__ R,
+                  const float* __restrict__ C, int N, int K, float* __restrict__ a, float* __restrict__ b,
+                  float* __restrict__ upart, const unsigned long long* __restrict__ cpart,
+                  unsigned int* __restrict__ done, const FinalArgs h, float* out) {
   dep_wait();
   dep_trigger();
   __shared__ float sh[kThreads / 32];
+  __shared__ double shd[kThreads / 32];
+  __shared__ unsigned long long shu[kThreads / 32];
+  __shared__ float an_s[kRowsPerSlab];
+  __shared__ bool last_s;
   const int k0 = blockIdx.x * kColsPerBlock + threadIdx.x * 4;
   const int n0 = blockIdx.y * kRowsPerSlab;
+  if (threadIdx.x < kRowsPerSlab && n0 + static_cast<int>(threadIdx.x) < N) {
+    const int n = n0 + threadIdx.x;
+    const float an = __fdiv_rn(1.0f, __fsqrt_rn(__fdiv_rn(R[n], out[0])));
+    an_s[threadIdx.x] = an;
+    if (blockIdx.x == 0) a[n] = an;
+  }
+  __syncthreads();
   float acc = 0.f;
   if (k0 < K) {
-    const float4 bk = *reinterpret_cast<const float4*>(b + k0);
+    const float4 c4 = *reinterpret_cast<const float4*>(C + k0);
+    const float4 bk = make_float4(
+        __fdiv_rn(1.0f, __fsqrt_rn(c4.x)), __fdiv_rn(1.0f, __fsqrt_rn(c4.y)),
+        __fdiv_rn(1.0f, __fsqrt_rn(c4.z)), __fdiv_rn(1.0f, __fsqrt_rn(c4.w)));
+    if (blockIdx.y == 0) *reinterpret_cast<float4*>(b + k0) = bk;
     for (int r0 = 0; r0 < kRowsPerSlab && n0 + r0 < N; r0 += kUnroll) {
       float4 g[kUnroll];
-      float an[kUnroll];
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
         const int n = n0 + r0 + u;
         g[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        an[u] = 0.f;
-        if (n < N) {
-          g[u] = __ldcs(reinterpret_cast<const float4*>(G + static_cast<int64_t>(n) * K + k0));
-          an[u] = a[n];
-        }
+        if (n < N) g[u] = __ldcs(reinterpret_cast<const float4*>(G + static_cast<int64_t>(n) * K + k0));
       }
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
-        const float u0 = af_u(g[u].x, an[u], bk.x), u1 = af_u(g[u].y, an[u], bk.y);
-        const float u2 = af_u(g[u].z, an[u], bk.z), u3 = af_u(g[u].w, an[u], bk.w);
+        if (n0 + r0 + u >= N) break;
+        const float an = an_s[r0 + u];
+        const float u0 = af_u(g[u].x, an, bk.x), u1 = af_u(g[u].y, an, bk.y);
+        const float u2 = af_u(g[u].z, an, bk.z), u3 = af_u(g[u].w, an, bk.w);
         acc += (u0 * u0 + u1 * u1) + (u2 * u2 + u3 * u3);
       }
     }
   }
   const float tot = block_sum(acc, sh);
-  if (threadIdx.x == 0) upart[static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x] = tot;
-}
-
-// One block: the step's scalars.  out = {Rbar (already there), step, decay,
-// rms_u, rms_x, alpha}.
-__global__ void __launch_bounds__(kThreads)
-    af_finalize_kernel(int N, int K, const float* __restrict__ upart,
-                       const unsigned long long* __restrict__ cpart, int nparts, float s_w,
-                       float rho, float eps2, float clip_d, int scale_parameter,
-                       float weight_decay, float* __restrict__ out) {
-  dep_wait();
-  dep_trigger();
-  __shared__ double shd[kThreads / 32];
-  __shared__ unsigned long long shu[kThreads / 32];
+  const int nparts = static_cast<int>(gridDim.x * gridDim.y);
+  if (threadIdx.x == 0) {
+    upart[static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x] = tot;
+    __threadfence();
+    last_s = atomicAdd(done, 1u) == static_cast<unsigned int>(nparts) - 1u;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!last_s) return;
   double us = 0.0;
   unsigned long long cs = 0;
-  for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
-    us += static_cast<double>(upart[i]);
+#pragma unroll 4
+  for (int i = threadIdx.x; i < nparts; i += kThreads) {
+    us += static_cast<double>(__ldcg(upart + i));
     cs += cpart[i];
   }
   us = block_sum(us, shd);
-  __syncthreads();
   cs = block_sum(cs, shu);
   if (threadIdx.x == 0) {
     const double nk = static_cast<double>(N) * static_cast<double>(K);
     const double rms_u = sqrt(us / nk);
-    const double rms_x = sqrt(static_cast<double>(cs) / nk) / static_cast<double>(s_w);
-    const double alpha =
-        static_cast<double>(rho) * (scale_parameter ? fmax(static_cast<double>(eps2), rms_x) : 1.0);
-    const double div = fmax(1.0, rms_u / static_cast<double>(clip_d));
-    out[1] = static_cast<float>(static_cast<double>(s_w) * alpha / div);
-    out[2] = static_cast<float>(1.0 - static_cast<double>(weight_decay) * alpha);
+    const double rms_x = sqrt(static_cast<double>(cs) / nk) / static_cast<double>(h.s_w);
+    const double alpha = static_cast<double>(h.rho) *
+                         (h.scale_parameter ? fmax(static_cast<double>(h.eps2), rms_x) : 1.0);
+    const double div = fmax(1.0, rms_u / static_cast<double>(h.clip_d));
+    out[1] = static_cast<float>(static_cast<double>(h.s_w) * alpha / div);
+    out[2] = static_cast<float>(1.0 - static_cast<double>(h.weight_decay) * alpha);
     out[3] = static_cast<float>(rms_u);
     out[4] = static_cast<float>(rms_x);
     out[5] = static_cast<float>(alpha);
@@ -265,13 +286,20 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 struct ApplyArgs {
-  int32_t qmin, qmax, round_mode;
-  uint32_t step_lo, tensor_id, key0, key1;
+  int32_t qmin, qmax;
+  PhiloxCall pc;
 };
 
-template <bool WIDE>  // WIDE: N * K >= 2^32, 64-bit index arithmetic
+// One group of four weights (one Philox block) per thread step.  Bound by
+// instruction issue (72 % of the slots; 69 MB take 10 us): the storage form and
+// the rounding mode are compiled in and the generator's per-call parts come
+// from the parameter space.  11.5 M weights 25.5 -> 20.6 us; a grid of all
+// groups in memory order, which suits the bandwidth-bound updates, 24.4.
+
+// WIDE: N * K >= 2^32, 64-bit index arithmetic; NEAREST: round_mode 1.
+template <bool WIDE, bool PACKED, bool NEAREST>
 __global__ void __launch_bounds__(kThreads)
-    af_apply_kernel(const float* __restrict__ G, int8_t* __restrict__ W, bool packed,
+    af_apply_kernel(const float* __restrict__ G, int8_t* __restrict__ W,
                     const float* __restrict__ fa, const float* __restrict__ fb,
                     const float* __restrict__ scal, int N, int K, const ApplyArgs a,
                     unsigned long long* changed) {
@@ -295,11 +323,11 @@ __global__ void __launch_bounds__(kThreads)
       k = static_cast<int>(e32 - static_cast<uint32_t>(n) * static_cast<uint32_t>(K));
     }
     const float4 g = __ldcs(reinterpret_cast<const float4*>(G + e));
+    const char4 cc = load_codes4(W, PACKED, e);
     const float4 b4 = *reinterpret_cast<const float4*>(fb + k);
     const float an = fa[n];
-    const char4 cc = load_codes4(W, packed, e);
     uint4 w = make_uint4(0, 0, 0, 0);
-    if (a.round_mode == 0) w = sr_words(static_cast<uint64_t>(gi), a.step_lo, a.tensor_id, a.key0, a.key1);
+    if (!NEAREST) w = philox_call(static_cast<uint64_t>(gi), a.pc);
     const float gs[4] = {g.x, g.y, g.z, g.w};
     const float bs[4] = {b4.x, b4.y, b4.z, b4.w};
     const int32_t c0[4] = {cc.x, cc.y, cc.z, cc.w};
@@ -309,27 +337,22 @@ __global__ void __launch_bounds__(kThreads)
     for (int j = 0; j < 4; ++j) {
       const float u = af_u(gs[j], an, bs[j]);
       const float x = __fsub_rn(__fmul_rn(static_cast<float>(c0[j]), decay), __fmul_rn(step, u));
-      r[j] = sr_round(x, ws[j], a.round_mode, a.qmin, a.qmax);
+      r[j] = sr_round(x, ws[j], NEAREST ? 1 : 0, a.qmin, a.qmax);
       n_changed += (r[j] != c0[j]);
     }
-    if (packed)
+    if (PACKED)
       Wp[gi] = static_cast<uint8_t>(tern_pack4(r[0], r[1], r[2], r[3]));
     else
       *reinterpret_cast<char4*>(W + e) =
           make_char4(static_cast<signed char>(r[0]), static_cast<signed char>(r[1]),
                      static_cast<signed char>(r[2]), static_cast<signed char>(r[3]));
   }
-  if (changed) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) n_changed += __shfl_xor_sync(0xffffffffu, n_changed, off);
-    if ((threadIdx.x & 31) == 0 && n_changed)
-      atomicAdd(changed, static_cast<unsigned long long>(n_changed));
-  }
+  if (changed) add_changed(changed, n_changed);
 }
 
 struct Layout {
   int nchunks, nslabs, gx, nparts;
-  size_t row_off, col_off, cpart_off, upart_off, scal_off, a_off, b_off, bytes;
+  size_t row_off, col_off, cpart_off, upart_off, scal_off, a_off, b_off, rsum_off, done_off, bytes;
 };
 
 size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
@@ -347,7 +370,9 @@ Layout layout(int64_t N, int64_t K) {
   L.scal_off = align256(L.upart_off + static_cast<size_t>(L.nparts) * 4);
   L.a_off = align256(L.scal_off + 8 * 4);
   L.b_off = align256(L.a_off + static_cast<size_t>(N) * 4);
-  L.bytes = align256(L.b_off + static_cast<size_t>(K) * 4);
+  L.rsum_off = align256(L.b_off + static_cast<size_t>(K) * 4);
+  L.done_off = align256(L.rsum_off + static_cast<size_t>((N + kThreads - 1) / kThreads) * 8);
+  L.bytes = L.done_off + 256;
   return L;
 }
 
@@ -374,25 +399,22 @@ int launch_adafactor_stats(const float* G, const int8_t* W, bool packed, float s
   float* colpart = reinterpret_cast<float*>(base + L.col_off);
   unsigned long long* cpart = reinterpret_cast<unsigned long long*>(base + L.cpart_off);
   float* upart = reinterpret_cast<float*>(base + L.upart_off);
-  float* scal = scalars_out;
   const int n = static_cast<int>(N), k = static_cast<int>(K);
+  double* rsum = reinterpret_cast<double*>(base + L.rsum_off);
+  unsigned int* done = reinterpret_cast<unsigned int*>(base + L.done_off);
   const dim3 grid(L.gx, L.nslabs);
   if (launch_dep(af_sq_partials_kernel, grid, kThreads, 0, stream, G, W, packed,
-                 h.scale_parameter != 0, n, k, h.eps1, rowpart, colpart, cpart))
+                 h.scale_parameter != 0, n, k, h.eps1, rowpart, colpart, cpart, done))
     return 3;
   const int row_blocks = (n + kThreads - 1) / kThreads;
   const int col_blocks = (k + 31) / 32;
   if (launch_dep(af_moments_kernel, row_blocks + col_blocks, kThreads, 0, stream, rowpart, colpart,
-                 L.nchunks, L.nslabs, n, k, row_blocks, h.b2, h.omb2, R, C))
+                 L.nchunks, L.nslabs, n, k, row_blocks, h.b2, h.omb2, R, C, rsum, done,
+                 scalars_out))
     return 3;
-  if (launch_dep(af_factors_kernel, (n + k + kThreads - 1) / kThreads, kThreads, 0, stream, R, C,
-                 n, k, a_out, b_out, scal))
-    return 3;
-  if (launch_dep(af_usq_partials_kernel, grid, kThreads, 0, stream, G, a_out, b_out, n, k,
-                 upart))
-    return 3;
-  return launch_dep(af_finalize_kernel, 1, kThreads, 0, stream, n, k, upart, cpart, L.nparts, s_w,
-                    h.rho, h.eps2, h.clip_d, h.scale_parameter, h.weight_decay, scal);
+  const FinalArgs fa = {s_w, h.rho, h.eps2, h.clip_d, h.weight_decay, h.scale_parameter};
+  return launch_dep(af_usq_kernel, grid, kThreads, 0, stream, G, R, C, n, k, a_out, b_out, upart,
+                    cpart, done + 1, fa, scalars_out);
 }
 
 int launch_adafactor_apply(const float* G, int8_t* W, bool packed, const float* fa,
@@ -402,11 +424,7 @@ int launch_adafactor_apply(const float* G, int8_t* W, bool packed, const float* 
   ApplyArgs a;
   a.qmin = uc.qmin;
   a.qmax = uc.qmax;
-  a.round_mode = uc.round_mode;
-  a.step_lo = uc.step_lo;
-  a.tensor_id = uc.tensor_id;
-  a.key0 = uc.key0;
-  a.key1 = uc.key1;
+  a.pc = philox_call_consts(uc);
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -414,12 +432,17 @@ int launch_adafactor_apply(const float* G, int8_t* W, bool packed, const float* 
   int64_t blocks = (groups + kThreads - 1) / kThreads;
   if (blocks > static_cast<int64_t>(sms) * 8) blocks = static_cast<int64_t>(sms) * 8;
   if (blocks < 1) blocks = 1;
-  if (N * K >= (int64_t(1) << 32))
-    return launch_dep(af_apply_kernel<true>, static_cast<int>(blocks), kThreads, 0, stream, G, W,
-                      packed, fa, fb, scalars, static_cast<int>(N), static_cast<int>(K), a,
-                      changed);
-  return launch_dep(af_apply_kernel<false>, static_cast<int>(blocks), kThreads, 0, stream, G, W,
-                    packed, fa, fb, scalars, static_cast<int>(N), static_cast<int>(K), a, changed);
+  const bool wide = N * K >= (int64_t(1) << 32), nearest = uc.round_mode == 1;
+  auto kern = packed ? (nearest ? (wide ? af_apply_kernel<true, true, true>
+                                        : af_apply_kernel<false, true, true>)
+                                : (wide ? af_apply_kernel<true, true, false>
+                                        : af_apply_kernel<false, true, false>))
+                     : (nearest ? (wide ? af_apply_kernel<true, false, true>
+                                        : af_apply_kernel<false, false, true>)
+                                : (wide ? af_apply_kernel<true, false, false>
+                                        : af_apply_kernel<false, false, false>));
+  return launch_dep(kern, static_cast<unsigned>(blocks), kThreads, 0, stream, G, W, fa, fb, scalars,
+                    static_cast<int>(N), static_cast<int>(K), a, changed);
 }
 
 }  // namespace dqt

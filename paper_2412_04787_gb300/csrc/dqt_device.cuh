@@ -496,6 +496,65 @@ __device__ __forceinline__ int32_t dqt_update_elem(const UpdateConsts& h, float 
   return sr_round(x, word, h.round_mode, h.qmin, h.qmax);
 }
 
+// Philox4x32-10 (the generator of sr_words) for the elements of one update
+// call: the round keys and, in the first round, the product of counter word
+// 2 (the step) and word 3 (the weight tensor) are the same for every
+// element, so the host computes them once (philox_call_consts).
+struct PhiloxCall {
+  uint32_t rk[20];  // rk[2r], rk[2r + 1]: round r's keys, key0 + r W0 and key1 + r W1
+  uint32_t c0x;     // hi(M1 * step) ^ rk[0]: round 0's first output word before ^ counter word 1
+  uint32_t c0y;     // lo(M1 * step): round 0's second output word
+  uint32_t x3k;     // tensor id ^ rk[1]
+};
+
+// The four Philox words of block `blk` (elements 4 blk .. 4 blk + 3), equal
+// to sr_words(blk, step, tensor id, key0, key1) of the call's constants.
+__device__ __forceinline__ uint4 philox_call(uint64_t blk, const PhiloxCall& k) {
+  const uint32_t x0 = static_cast<uint32_t>(blk), x1 = static_cast<uint32_t>(blk >> 32);
+  const uint64_t p0 = static_cast<uint64_t>(0xD2511F53u) * x0;
+  uint4 c = make_uint4(k.c0x ^ x1, k.c0y, static_cast<uint32_t>(p0 >> 32) ^ k.x3k,
+                       static_cast<uint32_t>(p0));
+#pragma unroll
+  for (int r = 1; r < 10; ++r) {
+    const uint64_t q0 = static_cast<uint64_t>(0xD2511F53u) * c.x;
+    const uint64_t q1 = static_cast<uint64_t>(0xCD9E8D57u) * c.z;
+    c = make_uint4(static_cast<uint32_t>(q1 >> 32) ^ c.y ^ k.rk[2 * r], static_cast<uint32_t>(q1),
+                   static_cast<uint32_t>(q0 >> 32) ^ c.w ^ k.rk[2 * r + 1], static_cast<uint32_t>(q0));
+  }
+  return c;
+}
+
+// The per-call Philox constants of PhiloxCall from the update constants.
+inline PhiloxCall philox_call_consts(const UpdateConsts& uc) {
+  PhiloxCall k{};
+  for (int r = 0; r < 10; ++r) {
+    k.rk[2 * r] = uc.key0 + static_cast<uint32_t>(r) * 0x9E3779B9u;
+    k.rk[2 * r + 1] = uc.key1 + static_cast<uint32_t>(r) * 0xBB67AE85u;
+  }
+  const uint64_t p1 = static_cast<uint64_t>(0xCD9E8D57u) * uc.step_lo;
+  k.c0x = static_cast<uint32_t>(p1 >> 32) ^ k.rk[0];
+  k.c0y = static_cast<uint32_t>(p1);
+  k.x3k = uc.tensor_id ^ k.rk[1];
+  return k;
+}
+
+// Adds the block's sum of n_changed to *changed: one atomic per block of 256
+// threads (a warp's each were 90000 on one address for an 11.5 M-weight
+// update in memory order, and took longer than the update).  All threads.
+__device__ __forceinline__ void add_changed(unsigned long long* changed, uint32_t n_changed) {
+  __shared__ uint32_t sh[8];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) n_changed += __shfl_xor_sync(0xffffffffu, n_changed, off);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = n_changed;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t n = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) n += sh[w];
+    if (n) atomicAdd(changed, static_cast<unsigned long long>(n));
+  }
+}
+
 // 2-bit packed ternary codes: code e of a tensor is field e % 4 (bits 2 (e % 4)
 // and up) of byte e / 4, a 2-bit two's-complement number (-1 = 3, 0, +1 = 1).
 __device__ __forceinline__ char4 tern_unpack4(uint32_t b) {

@@ -62,17 +62,6 @@ constexpr int kEpiWarps = 8;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr uint64_t kDrainNs = 1000000000ull;  // wait for in-flight copies/MMAs on abort
 
-// Philox4x32-10 (the generator of sr_words) for the elements of one update
-// call: the round keys and, in the first round, the product of counter word
-// 2 (the step) and word 3 (the weight tensor) are the same for every
-// element, so the host computes them once (philox_call_consts).
-struct PhiloxCall {
-  uint32_t rk[20];  // rk[2r], rk[2r + 1]: round r's keys, key0 + r W0 and key1 + r W1
-  uint32_t c0x;     // hi(M1 * step) ^ rk[0]: round 0's first output word before ^ counter word 1
-  uint32_t c0y;     // lo(M1 * step): round 0's second output word
-  uint32_t x3k;     // tensor id ^ rk[1]
-};
-
 struct Params {
   int M, N, Kred, num_kb, chunk_kb;
   int num_n, num_tiles;
@@ -485,23 +474,6 @@ __device__ __forceinline__ uint64_t l2_policy_evict_first() {
   uint64_t pol;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
   return pol;
-}
-
-// The four Philox words of block `blk` (elements 4 blk .. 4 blk + 3), equal
-// to sr_words(blk, step, tensor id, key0, key1) of the call's constants.
-__device__ __forceinline__ uint4 philox_call(uint64_t blk, const PhiloxCall& k) {
-  const uint32_t x0 = static_cast<uint32_t>(blk), x1 = static_cast<uint32_t>(blk >> 32);
-  const uint64_t p0 = static_cast<uint64_t>(0xD2511F53u) * x0;
-  uint4 c = make_uint4(k.c0x ^ x1, k.c0y, static_cast<uint32_t>(p0 >> 32) ^ k.x3k,
-                       static_cast<uint32_t>(p0));
-#pragma unroll
-  for (int r = 1; r < 10; ++r) {
-    const uint64_t q0 = static_cast<uint64_t>(0xD2511F53u) * c.x;
-    const uint64_t q1 = static_cast<uint64_t>(0xCD9E8D57u) * c.z;
-    c = make_uint4(static_cast<uint32_t>(q1 >> 32) ^ c.y ^ k.rk[2 * r], static_cast<uint32_t>(q1),
-                   static_cast<uint32_t>(q0 >> 32) ^ c.w ^ k.rk[2 * r + 1], static_cast<uint32_t>(q0));
-  }
-  return c;
 }
 
 template <bool PK>
@@ -1712,20 +1684,6 @@ int launch_pairs(const CUtensorMap& ta, const CUtensorMap& tb, Params p, cudaStr
 }
 
 }  // namespace
-
-// The per-call Philox constants of PhiloxCall from the update constants.
-static PhiloxCall philox_call_consts(const UpdateConsts& uc) {
-  PhiloxCall k{};
-  for (int r = 0; r < 10; ++r) {
-    k.rk[2 * r] = uc.key0 + static_cast<uint32_t>(r) * 0x9E3779B9u;
-    k.rk[2 * r + 1] = uc.key1 + static_cast<uint32_t>(r) * 0xBB67AE85u;
-  }
-  const uint64_t p1 = static_cast<uint64_t>(0xCD9E8D57u) * uc.step_lo;
-  k.c0x = static_cast<uint32_t>(p1 >> 32) ^ k.rk[0];
-  k.c0y = static_cast<uint32_t>(p1);
-  k.x3k = uc.tensor_id ^ k.rk[1];
-  return k;
-}
 
 // The arguments every GEMM kind takes from its launch record (the watchdog,
 // pointers, scales, update constants and images).

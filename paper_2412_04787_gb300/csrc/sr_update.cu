@@ -161,12 +161,7 @@ __global__ void __launch_bounds__(kThreads, SLABS ? 4 : 5)
     }
     if (packed) Wp[gi] = static_cast<uint8_t>(tern_pack4(pr[0], pr[1], pr[2], pr[3]));
   }
-  if (changed) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) n_changed += __shfl_xor_sync(0xffffffffu, n_changed, off);
-    if ((threadIdx.x & 31) == 0 && n_changed)
-      atomicAdd(changed, static_cast<unsigned long long>(n_changed));
-  }
+  if (changed) add_changed(changed, n_changed);
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -322,12 +317,7 @@ __global__ void __launch_bounds__(kThreads, 3)
         asm volatile("discard.global.L2 [%0], 128;" ::"l"(cur.src + s * sstride) : "memory");
     cur = nxt;
   }
-  if (changed) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) n_changed += __shfl_xor_sync(0xffffffffu, n_changed, off);
-    if ((threadIdx.x & 31) == 0 && n_changed)
-      atomicAdd(changed, static_cast<unsigned long long>(n_changed));
-  }
+  if (changed) add_changed(changed, n_changed);
 }
 
 // One group per thread, blocks in memory order (the kernels still stride, for
