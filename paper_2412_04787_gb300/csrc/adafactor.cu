@@ -63,7 +63,6 @@ __global__ void __launch_bounds__(kThreads, 4)
                           float* __restrict__ colpart, unsigned long long* __restrict__ cpart,
                           unsigned int* __restrict__ done) {
   dep_wait();
-  dep_trigger();
   __shared__ unsigned long long sh[kThreads / 32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int k0 = blockIdx.x * kColsPerBlock + threadIdx.x * 4;
@@ -134,7 +133,6 @@ __global__ void __launch_bounds__(kThreads)
                       float* __restrict__ R, float* __restrict__ C, double* __restrict__ rsum,
                       unsigned int* __restrict__ done, float* __restrict__ out) {
   dep_wait();
-  dep_trigger();
   if (static_cast<int>(blockIdx.x) < row_blocks) {
     __shared__ double shd[kThreads / 32];
     __shared__ bool last_s;
@@ -211,7 +209,6 @@ __global__ void __launch_bounds__(kThreads)
                   float* __restrict__ upart, const unsigned long long* __restrict__ cpart,
                   unsigned int* __restrict__ done, const FinalArgs h, float* out) {
   dep_wait();
-  dep_trigger();
   __shared__ float sh[kThreads / 32];
   __shared__ double shd[kThreads / 32];
   __shared__ unsigned long long shu[kThreads / 32];
@@ -304,7 +301,6 @@ __global__ void __launch_bounds__(kThreads)
                     const float* __restrict__ scal, int N, int K, const ApplyArgs a,
                     unsigned long long* changed) {
   dep_wait();
-  dep_trigger();
   const float step = scal[1], decay = scal[2];
   const int64_t ngroups = (static_cast<int64_t>(N) * K) >> 2;  // K % 4 == 0: no ragged group
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;

@@ -44,7 +44,6 @@ __global__ void __launch_bounds__(kRopeThreads)
     rope_kernel(const uint4* __restrict__ x, uint4* __restrict__ y, const float4* __restrict__ cs,
                 int64_t rows, int row_vecs, uint32_t S, int head_vecs, int R) {
   dep_wait();
-  dep_trigger();
   const int tr = row_vecs < kRopeThreads ? static_cast<int>(threadIdx.x) / row_vecs : 0;
   const int64_t row = static_cast<int64_t>(blockIdx.x) * R + tr;
   if (tr >= R || row >= rows) return;
@@ -120,7 +119,6 @@ __global__ void __launch_bounds__(kCeThreads)
     ce_fwd_kernel(const uint4* __restrict__ logits, const int64_t* __restrict__ tgt, int64_t V,
                   float* __restrict__ lse, float* __restrict__ row_loss) {
   dep_wait();
-  dep_trigger();
   __shared__ float sh_m[kCeThreads / 32], sh_s[kCeThreads / 32];
   constexpr float kLog2e = 1.44269504088896340736f;
   const int64_t r = blockIdx.x;
@@ -180,7 +178,6 @@ __global__ void __launch_bounds__(kCeThreads)
                   const float* __restrict__ lse, const float* __restrict__ scale, int64_t V,
                   uint4* __restrict__ dlogits) {
   dep_wait();
-  dep_trigger();
   const int64_t r = blockIdx.x;
   const int64_t nv = V >> 3;
   const int64_t t = tgt[r];
@@ -221,7 +218,6 @@ __global__ void __launch_bounds__(kEwThreads)
     swiglu_kernel(const uint4* __restrict__ g, const uint4* __restrict__ u, uint4* __restrict__ h,
                   int64_t nvec) {
   dep_wait();
-  dep_trigger();
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kEwThreads;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * kEwThreads + threadIdx.x; i < nvec;
        i += stride) {
@@ -245,7 +241,6 @@ __global__ void __launch_bounds__(kEwThreads)
                       const uint4* __restrict__ dh, uint4* __restrict__ dg,
                       uint4* __restrict__ du, int64_t nvec) {
   dep_wait();
-  dep_trigger();
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kEwThreads;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * kEwThreads + threadIdx.x; i < nvec;
        i += stride) {
@@ -284,7 +279,6 @@ __global__ void __launch_bounds__(32 * kNormWarps)
     rmsnorm_fwd_kernel(const uint4* __restrict__ x, const uint4* __restrict__ w, float eps,
                        int64_t rows, int nv, uint4* __restrict__ y, float* __restrict__ rstd) {
   dep_wait();
-  dep_trigger();
   const int lane = threadIdx.x & 31;
   const int64_t step = static_cast<int64_t>(gridDim.x) * kNormWarps;
   int64_t row = static_cast<int64_t>(blockIdx.x) * kNormWarps + (threadIdx.x >> 5);
@@ -367,7 +361,6 @@ __global__ void __launch_bounds__(32 * kNormBwdWarps, 1)
                        const float* __restrict__ rstd, const uint4* __restrict__ dy, int64_t rows,
                        int nv, uint4* __restrict__ dx, float* __restrict__ part) {
   dep_wait();
-  dep_trigger();
   constexpr int G = kNormBwdWarps / WPR;       // row groups per block
   __shared__ float4 sums[VPL * WPR * 64];      // one row of columns
   __shared__ float dots[2][G][WPR];            // the warps' parts of a row's sum, two rows in turn
@@ -490,7 +483,6 @@ __global__ void __launch_bounds__(32 * kNormBwdWarps, 1)
 __global__ void __launch_bounds__(1024)
     rmsnorm_dw_kernel(const float* __restrict__ part, int64_t P, int D, uint16_t* __restrict__ dw) {
   dep_wait();
-  dep_trigger();
   __shared__ float sh[32][33];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int col = blockIdx.x * 32 + lane;

@@ -33,7 +33,6 @@ __device__ __forceinline__ uint32_t pack_word(uint32_t w) {  // 4 int8 codes -> 
 __global__ void __launch_bounds__(kThreads)
     pack_kernel(const int8_t* __restrict__ c, int64_t n, uint8_t* __restrict__ out) {
   dep_wait();
-  dep_trigger();
   const int64_t nvec = n >> 4;  // 16 codes -> one 32-bit word of 4 bytes
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < nvec;
@@ -55,7 +54,6 @@ __global__ void __launch_bounds__(kThreads)
 __global__ void __launch_bounds__(kThreads)
     unpack_kernel(const uint8_t* __restrict__ p, int64_t n, int8_t* __restrict__ c) {
   dep_wait();
-  dep_trigger();
   const int64_t nvec = n >> 4;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < nvec;
@@ -92,7 +90,6 @@ __device__ __forceinline__ uint32_t tern_e4m3(uint32_t f) {
 __global__ void __launch_bounds__(kThreads)
     packed_to_bf16_kernel(const uint8_t* __restrict__ p, int64_t n, uint16_t* __restrict__ img) {
   dep_wait();
-  dep_trigger();
   const int64_t nvec = n >> 4;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < nvec;
@@ -114,7 +111,6 @@ __global__ void __launch_bounds__(kThreads)
 __global__ void __launch_bounds__(kThreads)
     packed_to_fp8_kernel(const uint8_t* __restrict__ p, int64_t n, uint8_t* __restrict__ out) {
   dep_wait();
-  dep_trigger();
   const int64_t nvec = n >> 4;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * kThreads;
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * kThreads + threadIdx.x; i < nvec;

@@ -73,7 +73,6 @@ __global__ void __launch_bounds__(kAqWarps * 32)
                      float* __restrict__ s_x, uint16_t* __restrict__ Xq_img,
                      uint16_t* __restrict__ Xdq) {
   dep_wait();
-  dep_trigger();
   const int row = blockIdx.x * kAqWarps + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= T) return;
@@ -428,7 +427,6 @@ __global__ void __launch_bounds__(256)
     codes_to_xdq_kernel(const int8_t* __restrict__ Xq, const float* __restrict__ s_x, int T,
                         int K, uint16_t* __restrict__ Xdq) {
   dep_wait();
-  dep_trigger();
   __shared__ uint16_t table[8][256];
   const int wid = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -481,7 +479,6 @@ __device__ __forceinline__ void codes16_to_bf16(const uint4 u, uint4& o0, uint4&
 __global__ void codes_to_bf16_kernel(const int8_t* __restrict__ W, int64_t numel,
                                      uint16_t* __restrict__ img) {
   dep_wait();
-  dep_trigger();
   const int64_t nvec = numel >> 4;  // 16-code vectors
   const int64_t nthr = static_cast<int64_t>(gridDim.x) * blockDim.x;
   const uint4* src = reinterpret_cast<const uint4*>(W);
@@ -525,7 +522,6 @@ __device__ __forceinline__ uint32_t codes4_to_e4m3(uint32_t w) {
 __global__ void codes_to_fp8_kernel(const int8_t* __restrict__ W, int64_t numel,
                                     uint8_t* __restrict__ out) {
   dep_wait();
-  dep_trigger();
   const int64_t nvec = numel >> 4;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
   const uint4* src = reinterpret_cast<const uint4*>(W);
@@ -549,7 +545,6 @@ __global__ void codes_to_fp8_kernel(const int8_t* __restrict__ W, int64_t numel,
 __global__ void codes_to_fp8_split_kernel(const int8_t* __restrict__ W, int64_t N, int64_t K,
                                           uint8_t* __restrict__ out) {
   dep_wait();
-  dep_trigger();
   const int64_t vpr = K >> 4;  // 16-code vectors per row
   const int64_t nvec = N * vpr;
   const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
