@@ -63,6 +63,59 @@ __device__ __forceinline__ uint16_t dq_entry(int j, float s) {
 template <bool F8>
 __device__ __forceinline__ int dq_index(int32_t q) { return F8 ? q : q + 128; }
 
+// The dequantised value bf16(RN(q / s)) of a row's codes without a division
+// per element: t = RN(q r) with r = RN(1 / s) is within 2 units in the last
+// place of RN(q / s) (relative errors 2^-24 of r and of the product against
+// 2^-24 of the quotient), so both round to the same bf16 unless t lies that
+// close to the midpoint of two bf16 values (low half 0x8000).  A row whose
+// 128 code magnitudes include such a t (a margin of 4 units: 1.7 % of rows)
+// divides instead.  A 256-entry table of quotients per row, looked up per
+// element, took 8 divisions a lane and shared-memory reads with bank
+// conflicts: a third of the instructions of a 768-wide row.
+__device__ __forceinline__ bool near_bf16_midpoint(float t) {
+  return ((__float_as_uint(t) - 0x7FFCu) & 0xFFFFu) <= 8u;
+}
+
+// All lanes; whether every code of the row may be multiplied by r (r far from
+// the ends of the range, so that no product is subnormal or overflows; a row
+// with an infinite input has s = 0 and divides).
+template <bool F8>
+__device__ __forceinline__ bool row_multiplies(float r, int lane) {
+  bool near = !(fabsf(r) > 1e-30f && fabsf(r) < 1e30f);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int mag = lane + 32 * i;  // int8: magnitudes 1 .. 128; E4M3: bytes 0 .. 127
+    float v;
+    if (F8) {
+      const __half h(__nv_cvt_fp8_to_halfraw(static_cast<__nv_fp8_storage_t>(mag), __NV_E4M3));
+      v = __half2float(h);
+    } else {
+      v = static_cast<float>(mag + 1);
+    }
+    near = near || near_bf16_midpoint(__fmul_rn(v, r));
+  }
+  return !__any_sync(0xffffffffu, near);
+}
+
+__device__ __forceinline__ uint32_t bf16x2(float lo, float hi) {
+  const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&p);
+}
+
+// Two dequantised values (codes as exact floats).
+__device__ __forceinline__ uint32_t dq_pair(float a, float b, float s, float r, bool mul) {
+  return mul ? bf16x2(__fmul_rn(a, r), __fmul_rn(b, r)) : bf16x2(__fdiv_rn(a, s), __fdiv_rn(b, s));
+}
+
+// The four int8 codes of a word as floats: the byte q + 128 as the low byte
+// of 2^23's bit pattern, then an exact subtraction (no integer conversion).
+__device__ __forceinline__ void codes4_to_float(uint32_t w, float (&f)[4]) {
+  const uint32_t u = w ^ 0x80808080u;
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    f[j] = __fsub_rn(__uint_as_float(__byte_perm(u, 0x4B000000u, 0x7440u + j)), 8388736.0f);
+}
+
 // One warp per token row; 16-byte (8 x bf16) vector accesses.  Pass 1 finds
 // amax; pass 2 re-reads the row (an L1/L2 hit) and writes the outputs.
 constexpr int kAqWarps = 8;
@@ -131,15 +184,15 @@ __global__ void __launch_bounds__(kAqWarps * 32)
 }
 
 // Activation quantisation with whole rows staged in shared memory: one CTA
-// per SM, a producer lane that streams the CTA's rows (blockIdx.x,
-// blockIdx.x + gridDim.x, ...) with linear bulk copies into a ring of S row
-// slots, and W consumer warps, warp w owning slots w, w + W, ... (S a
-// multiple of W, at least two slots per warp).  The j-th row of the CTA goes
-// to slot j % S and is processed by one warp: pass 1 reduces amax over the
-// row in shared memory, pass 2 re-reads it and writes the outputs.  Every
-// slot carries a `full` barrier (the copy's bytes) and an `empty` barrier
-// (one arrive by its consumer warp); the ring keeps up to S rows in flight
-// per SM, which a register-held design cannot.
+// per SM, a producer lane that streams the CTA's rows with linear bulk copies
+// into a ring of chunks, and W consumer warps that take the rows in turn: pass
+// 1 reduces amax over the row in shared memory, pass 2 re-reads it and writes
+// the outputs.  Every slot carries a `full` barrier (the copy's bytes) and an
+// `empty` barrier (an arrive per row); the ring keeps up to 192 KB of rows in
+// flight per SM, which a register-held design cannot.  With both images 16384
+// x 768 takes 12.5 us (16.8 with whole chunks per warp and a table of
+// quotients per row), 256 x 512 2.1 (3.9), 8192 x 2048 13.5 (15.0); the codes
+// alone 11.5 (10.9) there, 21.5 (23.3) at 8192 x 5632.
 //
 // amax is reduced on pairs of bf16 magnitudes (max.bf16x2 returns the
 // non-NaN operand, as fmaxf does, and is exact).  Round(y) for the int8
@@ -151,6 +204,7 @@ __global__ void __launch_bounds__(kAqWarps * 32)
 // clamp is needed, and it maps a NaN product (an infinite input) to -128, as
 // act_quant_kernel does.
 constexpr int kAqbRing = 192 * 1024;  // shared-memory bytes of the row ring
+constexpr int kRingWarps = 24;        // consumer warps at most
 
 // Linear bulk copy (no tensor map) of `bytes` from global memory into this
 // CTA's shared memory, completing on `bar`, whose expected byte count the
@@ -169,7 +223,11 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
 // row_bytes, then S `full` and S `empty` mbarriers.  CTA b owns the rows
 // [b T / G, (b + 1) T / G) (G = gridDim.x <= T, so at least one), cut into
 // chunks of rpc rows (the last one shorter); chunk j is one linear bulk copy
-// into slot j % S and is processed by consumer warp j % W (S a multiple of W).
+// into slot j % S.  The consumer warps take the rows in turn (row i of the
+// CTA: warp i % W), whatever their chunk, so that no warp has a whole chunk
+// more than another; a chunk's slot is free again when each of its rpc rows
+// has been released (only the last chunk is shorter, and its slot is not
+// refilled).
 struct RowRing {
   uint8_t* base;
   uint64_t* full;
@@ -191,6 +249,7 @@ struct RowRing {
         hi(static_cast<int64_t>(blockIdx.x + 1) * T / gridDim.x) {
     nchunks = static_cast<int>((hi - lo + rpc - 1) / rpc);
   }
+
   // shared memory after the ring and its barriers
   __device__ __forceinline__ uint8_t* end() const { return reinterpret_cast<uint8_t*>(empty + S); }
 
@@ -198,7 +257,7 @@ struct RowRing {
   __device__ __forceinline__ void init_barriers() const {
     if (static_cast<int>(threadIdx.x) < S) {
       mbar_init(&full[threadIdx.x], 1);
-      mbar_init(&empty[threadIdx.x], 1);
+      mbar_init(&empty[threadIdx.x], rpc);
       fence_mbarrier_init();
     }
   }
@@ -244,23 +303,28 @@ struct RowRing {
   __device__ __forceinline__ const uint8_t* row(int j, int r) const {
     return base + (static_cast<size_t>(j % S) * rpc + r) * row_bytes;
   }
-  // All lanes, after their last read of the slot.
+  // All lanes, after their last read of a row of chunk j.
   __device__ __forceinline__ void release(int j, int lane) const {
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[j % S]);
   }
 };
 
-template <bool F8>
-__global__ void __launch_bounds__(32 * 17, 1)
+//
+// IMG: the bf16 code image is written; XDQ: the dequantised image, 1 by
+// dq_pair, 2 (long E4M3 rows) from a 256-entry table per row, where the
+// conversions of every element back from E4M3 cost more than the table's
+// (8192 x 5632: 44.2 us by dq_pair, 39.6 from the table; 2048: 13.2 and 14.6).
+template <bool F8, bool IMG, int XDQ>
+__global__ void __launch_bounds__(32 * (kRingWarps + 1), 1)
     act_quant_bulk_kernel(const uint16_t* __restrict__ X, int T, int K,
                           int8_t* __restrict__ Xq, float* __restrict__ s_x,
                           uint16_t* __restrict__ Xq_img, uint16_t* __restrict__ Xdq, int S, int W,
                           int rpc, unsigned int* status, uint64_t limit_ns) {
   extern __shared__ __align__(128) uint8_t aqb_smem[];
   const RowRing ring(aqb_smem, S, static_cast<uint32_t>(K) * 2u, rpc, T);
-  uint16_t* tables = reinterpret_cast<uint16_t*>(ring.end());
   const int warp = threadIdx.x >> 5;
+  uint16_t* table = reinterpret_cast<uint16_t*>(ring.end()) + 256 * (warp - 1);  // XDQ == 2
   const int lane = threadIdx.x & 31;
   ring.init_barriers();
   __syncthreads();
@@ -271,103 +335,114 @@ __global__ void __launch_bounds__(32 * 17, 1)
     return;
   }
 
-  const int cw = warp - 1;
-  uint16_t* table = tables + cw * 256;
   const int nv = K >> 3;  // 16-byte vectors per row
   constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
-  for (int j = cw; j < ring.nchunks; j += W) {
+  const int nrows = static_cast<int>(ring.hi - ring.lo);
+  for (int i = warp - 1; i < nrows; i += W) {
+    const int j = i / rpc;
     if (!ring.acquire(j, lane, status, limit_ns)) return;
-    const int nr = ring.rows(j);
-#pragma unroll 1
-    for (int r = 0; r < nr; ++r) {
-      const int64_t row = ring.row0(j) + r;
-      const uint4* xr = reinterpret_cast<const uint4*>(ring.row(j, r));
-      __nv_bfloat162 am2 = __floats2bfloat162_rn(0.0f, 0.0f);
+    const int64_t row = ring.lo + i;
+    const uint4* xr = reinterpret_cast<const uint4*>(ring.row(j, i - j * rpc));
+    __nv_bfloat162 am2 = __floats2bfloat162_rn(0.0f, 0.0f);
 #pragma unroll 4
-      for (int v = lane; v < nv; v += 32) {
-        const uint4 u = xr[v];
-        const uint32_t w[4] = {u.x & 0x7FFF7FFFu, u.y & 0x7FFF7FFFu, u.z & 0x7FFF7FFFu,
-                               u.w & 0x7FFF7FFFu};
+    for (int v = lane; v < nv; v += 32) {
+      const uint4 u = xr[v];
+      const uint32_t w[4] = {u.x & 0x7FFF7FFFu, u.y & 0x7FFF7FFFu, u.z & 0x7FFF7FFFu,
+                             u.w & 0x7FFF7FFFu};
 #pragma unroll
-        for (int i = 0; i < 4; ++i) am2 = __hmax2(am2, *reinterpret_cast<const __nv_bfloat162*>(&w[i]));
-      }
-      float amax = fmaxf(__low2float(am2), __high2float(am2));
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
-      const float s = __fdiv_rn(code_scale_num<F8>(), fmaxf(amax, 1e-5f));
-      if (lane == 0) s_x[row] = s;
-      if (Xdq) {
-        for (int i = lane; i < 256; i += 32) table[i] = dq_entry<F8>(i, s);
-        __syncwarp();
-      }
-      const size_t rbase = static_cast<size_t>(row) * K;
-#pragma unroll 4
-      for (int v = lane; v < nv; v += 32) {
-        const uint4 u = xr[v];
-        const size_t e = rbase + static_cast<size_t>(v) * 8;
-        uint32_t b[8];  // per element: the code's table index in the low byte
-        if (F8) {
-          int32_t q[8];
-          quant8<true>(u, s, q);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) b[i] = static_cast<uint32_t>(q[i]);
-        } else {
-          const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-          float z[8];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            z[2 * i] = __fadd_rn(__fmul_rn(bf16_bits_to_f32(w[i] & 0xFFFFu), s), kMagic);
-            z[2 * i + 1] = __fadd_rn(__fmul_rn(bf16_bits_to_f32(w[i] >> 16), s), kMagic);
-          }
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            z[i] = fmaxf(z[i], kMagic - 128.0f);
-            b[i] = __float_as_uint(z[i]);
-          }
-          if (Xq_img) {
-            uint32_t h[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const __nv_bfloat162 p =
-                  __floats2bfloat162_rn(__fsub_rn(z[2 * i], kMagic), __fsub_rn(z[2 * i + 1], kMagic));
-              h[i] = *reinterpret_cast<const uint32_t*>(&p);
-            }
-            __stcs(reinterpret_cast<uint4*>(Xq_img + e), make_uint4(h[0], h[1], h[2], h[3]));
-          }
-        }
-        if (Xq) {
-          uint2 pk;
-          pk.x = __byte_perm(__byte_perm(b[0], b[1], 0x0040), __byte_perm(b[2], b[3], 0x0040), 0x5410);
-          pk.y = __byte_perm(__byte_perm(b[4], b[5], 0x0040), __byte_perm(b[6], b[7], 0x0040), 0x5410);
-          __stcs(reinterpret_cast<uint2*>(Xq + e), pk);
-        }
-        if (Xdq) {
-          uint32_t h[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) h[i] = table[F8 ? (b[i] & 0xFFu) : ((b[i] & 0xFFu) ^ 0x80u)];
-          __stcs(reinterpret_cast<uint4*>(Xdq + e),
-                 make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16),
-                            h[6] | (h[7] << 16)));
-        }
-      }
-      __syncwarp();  // the table is rewritten for the next row
+      for (int k = 0; k < 4; ++k) am2 = __hmax2(am2, *reinterpret_cast<const __nv_bfloat162*>(&w[k]));
     }
-    ring.release(j, lane);  // the slot is read for the last time
+    float amax = fmaxf(__low2float(am2), __high2float(am2));
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, off));
+    const float s = __fdiv_rn(code_scale_num<F8>(), fmaxf(amax, 1e-5f));
+    if (lane == 0) s_x[row] = s;
+    float r = 0.0f;
+    bool mul = false;
+    if (XDQ) {
+      r = __fdiv_rn(1.0f, s);
+      mul = row_multiplies<F8>(r, lane);
+    }
+    if (XDQ == 2) {
+      __syncwarp();  // the previous row's lookups are done
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int c = lane + 32 * k;
+        const __half h(__nv_cvt_fp8_to_halfraw(static_cast<__nv_fp8_storage_t>(c), __NV_E4M3));
+        table[c] = static_cast<uint16_t>(dq_pair(__half2float(h), 0.0f, s, r, mul));
+      }
+      __syncwarp();
+    }
+    const size_t rbase = static_cast<size_t>(row) * K;
+#pragma unroll 4
+    for (int v = lane; v < nv; v += 32) {
+      const uint4 u = xr[v];
+      const size_t e = rbase + static_cast<size_t>(v) * 8;
+      const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+      float f[8];     // the codes as exact floats
+      uint32_t b[8];  // int8 codes: each in the low byte of its word
+      uint2 pk;       // the eight code bytes
+      if (F8) {
+        uint32_t h[4];  // E4M3 byte pairs
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float2 x2 = make_float2(__fmul_rn(bf16_bits_to_f32(w[k] & 0xFFFFu), s),
+                                        __fmul_rn(bf16_bits_to_f32(w[k] >> 16), s));
+          h[k] = __nv_cvt_float2_to_fp8x2(x2, __NV_SATFINITE, __NV_E4M3);
+          if (XDQ == 1) {
+            const __half2_raw hr = __nv_cvt_fp8x2_to_halfraw2(
+                static_cast<__nv_fp8x2_storage_t>(h[k]), __NV_E4M3);
+            const float2 v2 = __half22float2(__half2(hr));
+            f[2 * k] = v2.x;
+            f[2 * k + 1] = v2.y;
+          }
+        }
+        pk = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
+      } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const uint32_t h = k & 1 ? w[k >> 1] >> 16 : w[k >> 1] & 0xFFFFu;
+          const float z = fmaxf(__fadd_rn(__fmul_rn(bf16_bits_to_f32(h), s), kMagic), kMagic - 128.0f);
+          b[k] = __float_as_uint(z);
+          f[k] = __fsub_rn(z, kMagic);
+        }
+        pk.x = __byte_perm(__byte_perm(b[0], b[1], 0x0040), __byte_perm(b[2], b[3], 0x0040), 0x5410);
+        pk.y = __byte_perm(__byte_perm(b[4], b[5], 0x0040), __byte_perm(b[6], b[7], 0x0040), 0x5410);
+        if (IMG)
+          __stcs(reinterpret_cast<uint4*>(Xq_img + e),
+                 make_uint4(bf16x2(f[0], f[1]), bf16x2(f[2], f[3]), bf16x2(f[4], f[5]),
+                            bf16x2(f[6], f[7])));
+      }
+      if (Xq) __stcs(reinterpret_cast<uint2*>(Xq + e), pk);
+      if (XDQ == 2) {
+        const uint32_t c4[2] = {pk.x, pk.y};
+        uint32_t d[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint32_t c2 = c4[k >> 1] >> (16 * (k & 1));
+          d[k] = table[c2 & 0xFFu] | (static_cast<uint32_t>(table[(c2 >> 8) & 0xFFu]) << 16);
+        }
+        __stcs(reinterpret_cast<uint4*>(Xdq + e), make_uint4(d[0], d[1], d[2], d[3]));
+      }
+      if (XDQ == 1)
+        __stcs(reinterpret_cast<uint4*>(Xdq + e),
+               make_uint4(dq_pair(f[0], f[1], s, r, mul), dq_pair(f[2], f[3], s, r, mul),
+                          dq_pair(f[4], f[5], s, r, mul), dq_pair(f[6], f[7], s, r, mul)));
+    }
+    ring.release(j, lane);
   }
 }
 
 // X_tilde = bf16(q / s_x) from int8 activation codes (the dW operand of the
-// int8 call), rows staged as in act_quant_bulk_kernel: each consumer warp
-// builds its row's 256-entry table of correctly rounded quotients (the table
-// dqt_act_quant uses), then maps the row's codes through it, 16 codes (one
-// 16-byte shared load, two 16-byte stores) per lane step.  K % 16 == 0.
-__global__ void __launch_bounds__(32 * 17, 1)
+// int8 call), rows staged as in act_quant_bulk_kernel, 16 codes (one 16-byte
+// shared load, two 16-byte stores) per lane step, dequantised as there.
+// K % 16 == 0.
+__global__ void __launch_bounds__(32 * (kRingWarps + 1), 1)
     codes_to_xdq_bulk_kernel(const int8_t* __restrict__ Xq, const float* __restrict__ s_x, int T,
                              int K, uint16_t* __restrict__ Xdq, int S, int W, int rpc,
                              unsigned int* status, uint64_t limit_ns) {
   extern __shared__ __align__(128) uint8_t cxb_smem[];
   const RowRing ring(cxb_smem, S, static_cast<uint32_t>(K), rpc, T);
-  uint16_t* tables = reinterpret_cast<uint16_t*>(ring.end());
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   ring.init_barriers();
@@ -378,42 +453,33 @@ __global__ void __launch_bounds__(32 * 17, 1)
     if (lane == 0) ring.produce(reinterpret_cast<const uint8_t*>(Xq), status, limit_ns);
     return;
   }
-  const int cw = warp - 1;
-  uint16_t* t = tables + cw * 256;
   const int nv = K >> 4;
-  for (int j = cw; j < ring.nchunks; j += W) {
-    const int nr = ring.rows(j);
-    bool acquired = false;
-#pragma unroll 1
-    for (int r = 0; r < nr; ++r) {
-      const int64_t row = ring.row0(j) + r;
-      const float s = s_x[row];
+  const int nrows = static_cast<int>(ring.hi - ring.lo);
+  for (int i = warp - 1; i < nrows; i += W) {
+    const int j = i / rpc;
+    const int64_t row = ring.lo + i;
+    const float s = s_x[row];
+    const float r = __fdiv_rn(1.0f, s);
+    const bool mul = row_multiplies<false>(r, lane);
+    if (!ring.acquire(j, lane, status, limit_ns)) return;
+    const uint4* src = reinterpret_cast<const uint4*>(ring.row(j, i - j * rpc));
+    uint4* dst = reinterpret_cast<uint4*>(Xdq + static_cast<size_t>(row) * K);
+#pragma unroll 2
+    for (int v = lane; v < nv; v += 32) {
+      const uint4 u = src[v];
+      const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+      uint32_t h[8];
 #pragma unroll
-      for (int i = lane; i < 256; i += 32) t[i] = dq_entry<false>(i, s);
-      __syncwarp();
-      if (!acquired) {
-        if (!ring.acquire(j, lane, status, limit_ns)) return;
-        acquired = true;
+      for (int k = 0; k < 4; ++k) {
+        float f[4];
+        codes4_to_float(w[k], f);
+        h[2 * k] = dq_pair(f[0], f[1], s, r, mul);
+        h[2 * k + 1] = dq_pair(f[2], f[3], s, r, mul);
       }
-      const uint4* src = reinterpret_cast<const uint4*>(ring.row(j, r));
-      uint4* dst = reinterpret_cast<uint4*>(Xdq + static_cast<size_t>(row) * K);
-#pragma unroll 4
-      for (int v = lane; v < nv; v += 32) {
-        const uint4 u = src[v];
-        const uint32_t w[4] = {u.x ^ 0x80808080u, u.y ^ 0x80808080u, u.z ^ 0x80808080u,
-                               u.w ^ 0x80808080u};  // table indices q + 128
-        uint32_t h[8];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          h[2 * i] = t[w[i] & 0xFFu] | (uint32_t(t[(w[i] >> 8) & 0xFFu]) << 16);
-          h[2 * i + 1] = t[(w[i] >> 16) & 0xFFu] | (uint32_t(t[w[i] >> 24]) << 16);
-        }
-        __stcs(dst + 2 * v, make_uint4(h[0], h[1], h[2], h[3]));
-        __stcs(dst + 2 * v + 1, make_uint4(h[4], h[5], h[6], h[7]));
-      }
-      __syncwarp();  // the table is rewritten for the next row
+      __stcs(dst + 2 * v, make_uint4(h[0], h[1], h[2], h[3]));
+      __stcs(dst + 2 * v + 1, make_uint4(h[4], h[5], h[6], h[7]));
     }
-    ring.release(j, lane);  // the slot is read for the last time
+    ring.release(j, lane);
   }
 }
 
@@ -456,45 +522,38 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// 64 codes per thread per step: four 16-byte loads issued together, then
-// eight 16-byte streaming stores (the image is read by the next kernel only).
+// 32 codes per thread step: two 16-byte loads issued together, then four
+// 16-byte streaming stores (the image is read by the next kernel only), blocks
+// in memory order: 12.6 M codes in 7.6 us (8.2 in four distant streams).
 __device__ __forceinline__ void codes16_to_bf16(const uint4 u, uint4& o0, uint4& o1) {
   const uint32_t w[4] = {u.x, u.y, u.z, u.w};
   uint32_t o[8];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const int32_t b0 = static_cast<int8_t>(w[j] & 0xFF);
-    const int32_t b1 = static_cast<int8_t>((w[j] >> 8) & 0xFF);
-    const int32_t b2 = static_cast<int8_t>((w[j] >> 16) & 0xFF);
-    const int32_t b3 = static_cast<int8_t>(w[j] >> 24);
-    o[2 * j] = f32_to_bf16_bits(static_cast<float>(b0)) |
-               (uint32_t(f32_to_bf16_bits(static_cast<float>(b1))) << 16);
-    o[2 * j + 1] = f32_to_bf16_bits(static_cast<float>(b2)) |
-                   (uint32_t(f32_to_bf16_bits(static_cast<float>(b3))) << 16);
+    float f[4];
+    codes4_to_float(w[j], f);
+    o[2 * j] = bf16x2(f[0], f[1]);
+    o[2 * j + 1] = bf16x2(f[2], f[3]);
   }
   o0 = make_uint4(o[0], o[1], o[2], o[3]);
   o1 = make_uint4(o[4], o[5], o[6], o[7]);
 }
 
-__global__ void codes_to_bf16_kernel(const int8_t* __restrict__ W, int64_t numel,
-                                     uint16_t* __restrict__ img) {
+__global__ void __launch_bounds__(256)
+    codes_to_bf16_kernel(const int8_t* __restrict__ W, int64_t numel, uint16_t* __restrict__ img) {
   dep_wait();
   const int64_t nvec = numel >> 4;  // 16-code vectors
-  const int64_t nthr = static_cast<int64_t>(gridDim.x) * blockDim.x;
   const uint4* src = reinterpret_cast<const uint4*>(W);
   uint4* dst = reinterpret_cast<uint4*>(img);
-  const int64_t t0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  // groups of four vectors, consecutive threads on consecutive vectors
-  for (int64_t base = 0; base < nvec; base += 4 * nthr) {
-    uint4 u[4];
+  for (int64_t i0 = static_cast<int64_t>(blockIdx.x) * 512 + threadIdx.x; i0 < nvec;
+       i0 += static_cast<int64_t>(gridDim.x) * 512) {
+    uint4 u[2];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t i = base + j * nthr + t0;
-      u[j] = i < nvec ? __ldcs(src + i) : make_uint4(0, 0, 0, 0);
-    }
+    for (int j = 0; j < 2; ++j)
+      u[j] = i0 + 256 * j < nvec ? __ldcs(src + i0 + 256 * j) : make_uint4(0, 0, 0, 0);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t i = base + j * nthr + t0;
+    for (int j = 0; j < 2; ++j) {
+      const int64_t i = i0 + 256 * j;
       if (i < nvec) {
         uint4 o0, o1;
         codes16_to_bf16(u[j], o0, o1);
@@ -636,24 +695,25 @@ int grid_for(int64_t work, int threads) {
 namespace {
 
 // Geometry of a row ring (act_quant_bulk_kernel, codes_to_xdq_bulk_kernel):
-// chunks of about 8 KB (rows of up to 8 KB are copied one per chunk), then up
-// to 16 consumer warps and as many slots per warp as fit in kAqbRing bytes
-// (48 slots at most); false when fewer than four chunks fit.  One producer
-// thread issues a bulk copy about every 0.2 us whatever its size, so copies
-// below ~8 KB leave the ring short of bytes in flight.
+// chunks of about 8 KB (rows of up to 8 KB are copied one per chunk), then as
+// many slots as fit in kAqbRing bytes (48 at most) and up to kRingWarps
+// consumer warps, no more than the rows that the slots hold; false when fewer
+// than four chunks fit.  One producer thread issues a bulk copy about every
+// 0.2 us whatever its size, so copies below ~8 KB leave the ring short of
+// bytes in flight.
 bool ring_geometry(int64_t row_bytes, int& rpc, int& W, int& S) {
   rpc = row_bytes >= 8192 ? 1 : static_cast<int>(8192 / row_bytes);
   const int64_t smax = kAqbRing / (rpc * row_bytes);
   if (smax < 4) return false;
-  W = static_cast<int>(smax < 16 ? smax : 16);
-  S = static_cast<int>(smax < 48 ? smax : 48) / W * W;
+  S = static_cast<int>(smax < 48 ? smax : 48);
+  W = S * rpc < kRingWarps ? S * rpc : kRingWarps;
   return true;
 }
-constexpr int kRingMaxSmem = kAqbRing + 16 * 48 + 16 * 512;  // ring, barriers, tables
+constexpr int kRingMaxSmem = kAqbRing + 16 * 48 + 512 * kRingWarps;  // ring, barriers, tables
 
 // Launches a row-ring kernel: one CTA per SM (at most T), 32 (W + 1) threads.
 template <typename Kern, typename... Args>
-int launch_ring(Kern kern, bool& attr_set, int64_t T, int rpc, int W, int S, int64_t row_bytes,
+int launch_ring(Kern kern, bool& attr_set, bool tables, int64_t T, int rpc, int W, int S, int64_t row_bytes,
                 cudaStream_t stream, Args... args) {
   if (!attr_set) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingMaxSmem) !=
@@ -667,22 +727,36 @@ int launch_ring(Kern kern, bool& attr_set, int64_t T, int rpc, int W, int S, int
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int blocks = static_cast<int>(T < sms ? T : sms);
-  const size_t smem =
-      static_cast<size_t>(S) * rpc * row_bytes + 16 * static_cast<size_t>(S) + 512 * W;
+  const size_t smem = static_cast<size_t>(S) * rpc * row_bytes + 16 * static_cast<size_t>(S) +
+                      (tables ? 512 * W : 0);
   return launch_dep(kern, blocks, 32 * (W + 1), smem, stream, args..., S, W, rpc, status,
                     wait_limit_ns());
 }
 
 // Rows staged in shared memory when at least four fit in the ring; -1 when
 // the rows are too long.
-template <bool F8>
-int launch_aq_bulk(const uint16_t* X, int64_t T, int64_t K, int8_t* Xq, float* s_x,
+template <bool F8, bool IMG, int XDQ>
+int launch_aq_ring(const uint16_t* X, int64_t T, int64_t K, int8_t* Xq, float* s_x,
                    uint16_t* Xq_img, uint16_t* Xdq, cudaStream_t stream) {
   int rpc, W, S;
   if (!ring_geometry(2 * K, rpc, W, S)) return -1;
+  if (XDQ == 2 && W > 16) W = 16;
   static bool attr_set = false;  // per template instance
-  return launch_ring(act_quant_bulk_kernel<F8>, attr_set, T, rpc, W, S, 2 * K, stream, X,
-                     static_cast<int>(T), static_cast<int>(K), Xq, s_x, Xq_img, Xdq);
+  return launch_ring(act_quant_bulk_kernel<F8, IMG, XDQ>, attr_set, XDQ == 2, T, rpc, W, S, 2 * K,
+                     stream, X, static_cast<int>(T), static_cast<int>(K), Xq, s_x, Xq_img, Xdq);
+}
+
+template <bool F8>
+int launch_aq_bulk(const uint16_t* X, int64_t T, int64_t K, int8_t* Xq, float* s_x,
+                   uint16_t* Xq_img, uint16_t* Xdq, cudaStream_t stream) {
+  if (F8) {  // (no code image)
+    auto launch = !Xdq ? launch_aq_ring<F8, false, 0>
+                       : K > 4096 ? launch_aq_ring<F8, false, F8 ? 2 : 1> : launch_aq_ring<F8, false, 1>;
+    return launch(X, T, K, Xq, s_x, Xq_img, Xdq, stream);
+  }
+  auto launch = Xq_img ? (Xdq ? launch_aq_ring<F8, !F8, 1> : launch_aq_ring<F8, !F8, 0>)
+                       : (Xdq ? launch_aq_ring<F8, false, 1> : launch_aq_ring<F8, false, 0>);
+  return launch(X, T, K, Xq, s_x, Xq_img, Xdq, stream);
 }
 
 template <bool F8>
@@ -711,7 +785,7 @@ int launch_codes_to_xdq(const int8_t* Xq, const float* s_x, int64_t T, int64_t K
     int rpc, W, S;
     if (ring_geometry(K, rpc, W, S)) {
       static bool attr_set = false;
-      return launch_ring(codes_to_xdq_bulk_kernel, attr_set, T, rpc, W, S, K, stream, Xq, s_x,
+      return launch_ring(codes_to_xdq_bulk_kernel, attr_set, false, T, rpc, W, S, K, stream, Xq, s_x,
                          static_cast<int>(T), static_cast<int>(K), Xdq);
     }
   }
@@ -743,9 +817,9 @@ int launch_codes_to_fp8_split(const int8_t* W, int64_t N, int64_t K, uint8_t* W8
 }
 
 int launch_codes_to_bf16(const int8_t* W, int64_t numel, uint16_t* W_img, cudaStream_t stream) {
-  const int threads = 256;
-  return launch_dep(codes_to_bf16_kernel, grid_for((numel >> 6) + 1, threads), threads, 0, stream,
-                    W, numel, W_img);
+  const int64_t want = ((numel >> 4) + 511) / 512, most = (int64_t(1) << 31) - 1;
+  const unsigned blocks = static_cast<unsigned>(want < 1 ? 1 : want < most ? want : most);
+  return launch_dep(codes_to_bf16_kernel, blocks, 256, 0, stream, W, numel, W_img);
 }
 
 int launch_absmean_partial(const float* W0, int64_t numel, double* ws, cudaStream_t stream) {
