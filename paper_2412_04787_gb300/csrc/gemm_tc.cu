@@ -903,6 +903,62 @@ struct SmemPair {
   static_assert((2 * STAGES + 5) * 8 + 4 <= 176, "barrier area: barriers, then the update constants");
 };
 
+// The last slice of a drained forward's tail region (two 32 x 32 blocks of one
+// warp): the slices' int32 partials added and the output written.
+template <int NB>
+__device__ __forceinline__ void drain_slices(const CUtensorMap& map, OutStage<NB>& out,
+                                             const Params& p, int lane, int row0, int nbase,
+                                             float a_t, const int32_t* blk, long long sstride) {
+#pragma unroll 1
+  for (int cc = 0; cc < 2; ++cc) {
+    const int32_t* src0 = blk + cc * 1024;
+    int32_t sum[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) sum[i] = 0;
+#pragma unroll 1
+    for (int sl = 0; sl < p.tail_splits; ++sl)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int4 v = __ldcg(reinterpret_cast<const int4*>(src0 + sl * sstride) + 32 * j + lane);
+        sum[4 * j] += v.x;
+        sum[4 * j + 1] += v.y;
+        sum[4 * j + 2] += v.z;
+        sum[4 * j + 3] += v.w;
+      }
+    __syncwarp();
+#pragma unroll 1
+    for (int sl = 0; sl < p.tail_splits; ++sl) l2_discard_line(src0 + sl * sstride + lane * 32);
+    const int gn0 = nbase + 32 * cc;
+    if (gn0 < p.N && row0 < p.M)  // warp-uniform
+      out_block_int(map, out, p, lane, row0, gn0, a_t, sum);
+  }
+}
+
+// One warp's region of a tail slice is stored (all lanes): counts it, and
+// returns whether it was the last of the tile's slices there, in which case
+// the other slices' partials are visible.
+__device__ __forceinline__ bool tail_last(const Params& q, int jt, int rank, int warps, int w,
+                                          int lane) {
+  __threadfence();
+  __syncwarp();
+  unsigned long long done = 0;
+  if (lane == 0) {
+    unsigned long long* ctr = q.tail_ctr + (static_cast<long long>(jt) * 2 + rank) * warps + w;
+    unsigned long long assumed = 0ull, nv;
+    while (true) {  // at most tail_splits + 1 tries: each failure sees another slice's count
+      nv = (assumed >> 16) == q.tail_tag ? assumed + 1ull : ((q.tail_tag << 16) | 1ull);
+      const unsigned long long prev = atomicCAS(ctr, assumed, nv);
+      if (prev == assumed) break;
+      assumed = prev;
+    }
+    done = nv & 0xFFFFull;
+  }
+  done = __shfl_sync(0xffffffffu, done, 0);
+  if (done != static_cast<unsigned long long>(q.tail_splits)) return false;
+  __threadfence();
+  return true;
+}
+
 // DR (forward only): every chunk of chunk_kb k-blocks is accumulated on its
 // own (an exact fp32 integer sum) in the two alternating accumulators, and
 // the epilogue warps fold each chunk into running int32 sums held in their
@@ -1149,6 +1205,10 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
     float4* xp = reinterpret_cast<float4*>(smem + S::XPOSE_OFF + (warp - 2) * kGradBytes);  // dW
     OutStage<S::OUT_NB> out{smem + S::XPOSE_OFF + (warp - 2) * S::OUT_NB * kOutBytes, 0};
     uint32_t n_changed = 0, n_changed2 = 0;  // changed codes of p's and p2's units
+    // DR: the tail tile whose region this warp finished last, its slices to be
+    // added after the unit loop (a cluster's slice is its last unit: there are
+    // no more slices than clusters), where the running sums are dead
+    int drain_tile = -1;
     int u = 0;
     bool ok = true;
     DwRow st[4];            // dW: optimiser state of the half-chunk being updated
@@ -1173,7 +1233,7 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
       }
       if (DR) {
         static_assert(!DR || HALF == 64, "two 32-column chunks of running sums per lane");
-        const int nchunks = (q.num_kb + q.chunk_kb - 1) / q.chunk_kb;
+        const int nchunks = (un.kb1 - un.kb0 + q.chunk_kb - 1) / q.chunk_kb;
         int32_t run0[32], run1[32];
         for (int c = 0; c < nchunks; ++c, ++u) {
           const int b = u & 1;
@@ -1198,11 +1258,28 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
           if (lane == 0) mbar_arrive_cluster(acc_empty_lead + 8u * b);
         }
         if (!ok) return false;
+        --u;  // the loop header counts one unit per tile
+        if (un.slice >= 0) {
+          // a tail slice, as below, with int32 partials (a slice's sums may
+          // pass 2^24)
+          const int jt = tile - q.full_tiles;
+          const long long sstride = static_cast<long long>(q.tail_tiles) * 65536LL;
+          int32_t* blk = reinterpret_cast<int32_t*>(q.part) + static_cast<long long>(jt) * 65536LL +
+                         ((static_cast<int>(rank) * 4 + quad) * 8 + half * (HALF / 32)) * 1024;
+          int4* dst = reinterpret_cast<int4*>(blk + un.slice * sstride) + lane;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            __stcg(dst + 32 * j, make_int4(run0[4 * j], run0[4 * j + 1], run0[4 * j + 2], run0[4 * j + 3]));
+            __stcg(dst + 256 + 32 * j,
+                   make_int4(run1[4 * j], run1[4 * j + 1], run1[4 * j + 2], run1[4 * j + 3]));
+          }
+          if (tail_last(q, jt, static_cast<int>(rank), EW, warp - 2, lane)) drain_tile = tile;
+          return true;
+        }
         if (gm - lane < q.M) {
           if (nbase < q.N) out_block_int(tmD, out, q, lane, gm - lane, nbase, a_t, run0);
           if (nbase + 32 < q.N) out_block_int(tmD, out, q, lane, gm - lane, nbase + 32, a_t, run1);
         }
-        --u;  // the loop header counts one unit per tile
         return true;
       }
       const int b = u & 1;
@@ -1266,24 +1343,7 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(acc_empty_lead + 8u * b);  // accumulator released
-          __threadfence();
-          __syncwarp();
-          unsigned long long done = 0;
-          if (lane == 0) {
-            unsigned long long* ctr =
-                q.tail_ctr + (static_cast<long long>(jt) * 2 + rank) * EW + (warp - 2);
-            unsigned long long assumed = 0ull, nv;
-            while (true) {  // at most tail_splits + 1 tries: each failure sees another slice's count
-              nv = (assumed >> 16) == q.tail_tag ? assumed + 1ull : ((q.tail_tag << 16) | 1ull);
-              const unsigned long long prev = atomicCAS(ctr, assumed, nv);
-              if (prev == assumed) break;
-              assumed = prev;
-            }
-            done = nv & 0xFFFFull;
-          }
-          done = __shfl_sync(0xffffffffu, done, 0);
-          if (done == static_cast<unsigned long long>(q.tail_splits)) {
-            __threadfence();
+          if (tail_last(q, jt, static_cast<int>(rank), EW, warp - 2, lane)) {
             const float* src0 = q.part + static_cast<long long>(jt) * 65536LL + blk0;
             const long long sstride = static_cast<long long>(q.tail_tiles) * 65536LL;
 #pragma unroll 1
@@ -1364,6 +1424,19 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
     for (int t = cid; t < total && ok; t += ncl, ++u)
       ok = (GRP && t >= p.num_tiles) ? epi_unit(p2, t - p.num_tiles, n_changed2)
                                      : epi_unit(p, t, n_changed);
+    if (DR && drain_tile >= 0) {
+      const int row0 = pair_tile_m(p, drain_tile) * 256 + static_cast<int>(rank) * 128 + quad * 32;
+      const int col0 = pair_tile_n(p, drain_tile) * BN;
+      float a_t = 0.0f;
+      if (row0 + lane < p.M)
+        a_t = __fdiv_rn(1.0f, __fmul_rn(p.s_x[row0 + lane],
+                                        p.split > 0 && col0 >= p.split ? p.scale1 : p.scale));
+      drain_slices(tmD, out, p, lane, row0, col0 + half * HALF, a_t,
+                   reinterpret_cast<const int32_t*>(p.part) +
+                       static_cast<long long>(drain_tile - p.full_tiles) * 65536LL +
+                       ((static_cast<int>(rank) * 4 + quad) * 8 + half * (HALF / 32)) * 1024,
+                   static_cast<long long>(p.tail_tiles) * 65536LL);
+    }
     if (!ok && lane == 0) record_timeout(p.status);
     if (lane == 0) bulk_wait_read<0>();  // this warp's stores have read shared memory
     if (EPI == GEMM_DW && p.changed) {
@@ -1528,8 +1601,9 @@ TailPlan tail_plan(int M, int N, int Kred, int clusters) {
 }
 
 // Forward / dX tail workspace: the slice counters (2 CTA ranks x 8 epilogue
-// warps per tail tile, tail <= clusters) in the first kTailCtrBytes, then the
-// partials (tail * splits <= clusters tiles of 256 x 256 floats).
+// warps, 16 with drained chunks, per tail tile) in the first kTailCtrBytes,
+// then the partials (tail * splits <= clusters tiles of 256 x 256 floats, or
+// int32 sums).
 constexpr size_t kTailCtrBytes = 16384;
 
 // The tail partials start on a 256-byte boundary inside the workspace (the
@@ -1544,6 +1618,8 @@ static float* tail_partials(void* ws, size_t ctr) {
 // least 4096 long: a slice's fixed costs (its pipeline fill, the partials'
 // round trip through L2, the fix-up) are ~10 us, which a cut of a 2048-long
 // reduction (~12 us of tile) does not win back.
+// Drained 8-bit forwards gain as the others: 8192 x 5632 -> 2048 (256 tiles:
+// 3.37 waves) 110.0 -> 105.6 us with int32 partials.
 constexpr int kTailMinKb = 4096 / BK;
 
 size_t gemm_tail_bytes(int M, int N, int Kred) {
@@ -1638,15 +1714,16 @@ int launch_pairs(const CUtensorMap& ta, const CUtensorMap& tb, Params p, cudaStr
   p.tail_kbps = p.num_kb;
   p.part = nullptr;
   if (plan) *plan = TailPlan{0, 0, 0, 0, 0};
-  if ((EPI == GEMM_DW || ((EPI == GEMM_FWD || EPI == GEMM_DX) && !DR && p.num_kb >= kTailMinKb)) &&
+  if ((EPI == GEMM_DW || ((EPI == GEMM_FWD || EPI == GEMM_DX) && p.num_kb >= kTailMinKb)) &&
       tail_ws && plan && p.splits == 1) {
     const TailPlan tp = tail_plan(p.M, p.N, p.Kred, max_clusters);
     const size_t ctr = EPI == GEMM_DW ? 0 : kTailCtrBytes;
-    static_assert(2 * 8 * 8 * 128 <= kTailCtrBytes, "slice counters: 128 tail tiles");
+    // the slice counters' room: one per tail tile, CTA and epilogue warp
+    constexpr int kCtrTiles = static_cast<int>(kTailCtrBytes / (2 * 8 * PairCfg<EPI, DR>::EW));
     float* part = tail_partials(tail_ws, ctr);
     const size_t used = static_cast<size_t>(reinterpret_cast<uint8_t*>(part) -
                                             static_cast<uint8_t*>(tail_ws)) + tp.bytes;
-    if (tp.splits >= 2 && tp.tail <= 128 && used <= tail_ws_bytes) {
+    if (tp.splits >= 2 && (EPI == GEMM_DW || tp.tail <= kCtrTiles) && used <= tail_ws_bytes) {
       p.full_units = tp.full;
       p.full_tiles = tp.full;
       p.tail_tiles = tp.tail;
@@ -1764,8 +1841,11 @@ int launch_gemm(const GemmLaunch& g, cudaStream_t stream) {
       if (!make_map(&ta, g.A, g.Kred, g.M, BK, BM)) return 3;
       if (drain) {
         if (!make_map(&tb, g.B, g.Kred, g.N, BK, 128)) return 3;
-        if (gemm_mode() == 0)
-          return launch_pairs<false, false, GEMM_FWD, false, true>(ta, tb, p, stream);
+        if (gemm_mode() == 0) {
+          TailPlan tp{0, 0, 0, 0, 0};
+          return launch_pairs<false, false, GEMM_FWD, false, true>(
+              ta, tb, p, stream, g.ws, g.ws_bytes, g.ws ? &tp : nullptr);
+        }
         return launch_tiles<128, false, false, GEMM_FWD, true>(ta, tb, p, stream);
       }
       if (!make_map(&tb, g.B, g.Kred, g.N, BK, g2.pair ? 128 : 256)) return 3;
