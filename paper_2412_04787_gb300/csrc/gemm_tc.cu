@@ -884,11 +884,11 @@ struct PairCfg {
   static constexpr int THREADS = 64 + 32 * EW;
 };
 
-template <int EPI, bool DR = false>
+template <int EPI, bool DR = false, int BN = 256>
 struct SmemPair {
   static constexpr int EW = PairCfg<EPI, DR>::EW;
   static constexpr int A_BYTES = 128 * BK * 2;
-  static constexpr int B_BYTES = 128 * BK * 2;  // this CTA's half of the B tile
+  static constexpr int B_BYTES = BN / 2 * BK * 2;  // this CTA's half of the B tile
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int STAGES = (EPI == GEMM_DW) ? 5 : 6;
   static constexpr int XPOSE_OFF = STAGES * STAGE_BYTES;
@@ -970,22 +970,22 @@ __device__ __forceinline__ bool tail_last(const Params& q, int jt, int rank, int
 // GRP: one launch for two dW problems over the same reduction length: p's
 // units, then p2's (tensor maps tmA2, tmB2), each with its own shape,
 // optimiser state, images, constants and tile order; whole tiles only.
-template <bool A_MN, bool B_MN, int EPI, bool PK, bool DR, bool UCD, bool GRP>
+// BN: width of the output tile (256; 128 for outputs of few tiles, see pair_bn).
+template <bool A_MN, bool B_MN, int EPI, bool PK, bool DR, bool UCD, bool GRP, int BN>
 __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUtensorMap& tmB,
                                                const CUtensorMap& tmD, const CUtensorMap& tmP,
                                                const Params& p, const CUtensorMap& tmA2,
                                                const CUtensorMap& tmB2, const Params& p2) {
-  using S = SmemPair<EPI, DR>;
+  using S = SmemPair<EPI, DR, BN>;
   static_assert(!DR || EPI == GEMM_FWD, "drained chunks: exact integer forward only");
   static_assert(!GRP || (EPI == GEMM_DW && !DR && !UCD), "grouped launches: dW, constants by value");
   constexpr int ST = S::STAGES;
   constexpr int EW = S::EW;
-  constexpr int BN = 256;           // pair tile width; each CTA holds all 256 columns of its rows
-  constexpr int HALF = BN / (EW / 4);  // columns per epilogue warp
+  constexpr int HALF = BN / (EW / 4);  // columns per epilogue warp (a CTA holds all BN of its rows)
   constexpr bool F8 = EPI == GEMM_FWD8;
   constexpr int KB = F8 ? 128 : BK;  // reduction elements per stage (one 128-byte row)
   static_assert(!F8 || (!A_MN && !B_MN), "E4M3 operands are read K-major");
-  constexpr uint32_t IDESC = F8 ? idesc_e4m3(256, 256) : idesc_bf16(256, 256, A_MN, B_MN);
+  constexpr uint32_t IDESC = F8 ? idesc_e4m3(256, BN) : idesc_bf16(256, BN, A_MN, B_MN);
   constexpr uint32_t TMEM_COLS = 512;
   constexpr uint32_t MN_CHUNK_BYTES = 64 * BK * 2;
 
@@ -1065,7 +1065,7 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
         const Unit un = decode_unit(q, tl);
         const int tile = un.tile, kb0 = un.kb0, kb1 = un.kb1;
         const int m0 = pair_tile_m(q, tile) * 256 + static_cast<int>(rank) * 128;
-        const int n0 = pair_tile_n(q, tile) * BN + static_cast<int>(rank) * 128;
+        const int n0 = pair_tile_n(q, tile) * BN + static_cast<int>(rank) * (BN / 2);
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
           if (it >= ST && !mbar_wait_cl(&empty[s], ph ^ 1u, q.wait_ns)) return false;
           if (leader) mbar_arrive_expect_tx(&full[s], 2 * S::STAGE_BYTES);
@@ -1097,11 +1097,11 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
             // X~ (all K columns) is re-read by every wave of output-row tiles,
             // while each dY column block is read by one wave: keep X~ in L2
 #pragma unroll
-            for (int j = 0; j < 2; ++j)
+            for (int j = 0; j < BN / 128; ++j)
               tma_load_2d_pair_hint(&B, bar, b + j * MN_CHUNK_BYTES, n0 + 64 * j, k0, pol_b);
           } else {
 #pragma unroll
-            for (int j = 0; j < 2; ++j)
+            for (int j = 0; j < BN / 128; ++j)
               tma_load_2d_pair(&B, bar, b + j * MN_CHUNK_BYTES, n0 + 64 * j, k0);
           }
           if (++s == ST) {
@@ -1461,13 +1461,14 @@ __device__ __forceinline__ void gemm_pair_body(const CUtensorMap& tmA, const CUt
   }
 }
 
-template <bool A_MN, bool B_MN, int EPI, bool PK = false, bool DR = false, bool UCD = false>
+template <bool A_MN, bool B_MN, int EPI, bool PK = false, bool DR = false, bool UCD = false,
+          int BN = 256>
 __global__ void __launch_bounds__(PairCfg<EPI, DR>::THREADS, 1)
     gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA,
                      const __grid_constant__ CUtensorMap tmB,
                      const __grid_constant__ CUtensorMap tmD,
                      const __grid_constant__ CUtensorMap tmP, const __grid_constant__ Params p) {
-  gemm_pair_body<A_MN, B_MN, EPI, PK, DR, UCD, false>(tmA, tmB, tmD, tmP, p, tmA, tmB, p);
+  gemm_pair_body<A_MN, B_MN, EPI, PK, DR, UCD, false, BN>(tmA, tmB, tmD, tmP, p, tmA, tmB, p);
 }
 
 // Two dW + update problems in one persistent launch (both operands MN-major,
@@ -1478,8 +1479,8 @@ __global__ void __launch_bounds__(PairCfg<GEMM_DW, false>::THREADS, 1)
                          const __grid_constant__ CUtensorMap tmA2,
                          const __grid_constant__ CUtensorMap tmB2,
                          const __grid_constant__ Params p2) {
-  gemm_pair_body<true, true, GEMM_DW, false, false, false, true>(tmA, tmB, tmA, tmA, p, tmA2, tmB2,
-                                                                 p2);
+  gemm_pair_body<true, true, GEMM_DW, false, false, false, true, 256>(tmA, tmB, tmA, tmA, p, tmA2,
+                                                                      tmB2, p2);
 }
 
 // ---------------------------------------------------------------------------
@@ -1566,7 +1567,8 @@ int launch_tiles(const CUtensorMap& ta, const CUtensorMap& tb, Params p, cudaStr
   return launch_dep(kern, grid, kThreads, smem, stream, ta, tb, p);
 }
 
-template <bool A_MN, bool B_MN, int EPI, bool PK = false, bool DR = false, bool UCD = false>
+template <bool A_MN, bool B_MN, int EPI, bool PK = false, bool DR = false, bool UCD = false,
+          int BN = 256>
 int launch_pairs(const CUtensorMap& ta, const CUtensorMap& tb, Params p, cudaStream_t stream,
                  void* tail_ws = nullptr, size_t tail_ws_bytes = 0, TailPlan* plan = nullptr);
 
@@ -1658,6 +1660,20 @@ int dw_splits(int M, int N, int Kred) {
 
 namespace {
 
+// Width of the 2-SM tiles of an M x N output cut into `splits` slices: 128
+// where even the narrow tiles give each SM pair at most one unit of work. The
+// launch is then one tile long, and half a tile has half the epilogue and
+// spreads over twice the SMs (its k-blocks take as long: ~530 cycles at either
+// width, and with two more stages in flight). 256 x 512 x 512, replayed:
+// forward 6.6 -> 5.8 us, dX 6.4 -> 5.7, weight gradient and update 9.2 -> 8.1.
+int pair_bn(int M, int N, int splits) {
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const long long units = static_cast<long long>((M + 255) / 256) * ((N + 127) / 128) * splits;
+  return units <= sms / 2 ? 128 : 256;
+}
+
 // Launches that cut their last wave with slice counters (all GEMM kinds).
 std::atomic<unsigned long long> g_tail_launches{0};
 
@@ -1665,21 +1681,21 @@ std::atomic<unsigned long long> g_tail_launches{0};
 // 256-wide panels is the one re-read by every wave (and kept in L2): X_tilde
 // (along the rows) when the output has more row tiles, dY (down the columns)
 // when it has more column tiles.
-void pair_tiling(Params& p, bool dw) {
-  p.num_n = (p.N + 255) / 256;
+void pair_tiling(Params& p, bool dw, int bn = 256) {
+  p.num_n = (p.N + bn - 1) / bn;
   p.num_m = (p.M + 255) / 256;
   p.num_tiles = p.num_m * p.num_n * p.splits;
   p.col_major = dw && p.num_n > p.num_m;
 }
 
-template <bool A_MN, bool B_MN, int EPI, bool PK, bool DR, bool UCD>
+template <bool A_MN, bool B_MN, int EPI, bool PK, bool DR, bool UCD, int BN>
 int launch_pairs(const CUtensorMap& ta, const CUtensorMap& tb, Params p, cudaStream_t stream,
                  void* tail_ws, size_t tail_ws_bytes, TailPlan* plan) {
-  auto kern = gemm_pair_kernel<A_MN, B_MN, EPI, PK, DR, UCD>;
-  const int smem = SmemPair<EPI, DR>::BYTES;
+  auto kern = gemm_pair_kernel<A_MN, B_MN, EPI, PK, DR, UCD, BN>;
+  const int smem = SmemPair<EPI, DR, BN>::BYTES;
   constexpr int threads = PairCfg<EPI, DR>::THREADS;
   static int max_clusters = 0;  // per template instance
-  pair_tiling(p, EPI == GEMM_DW);
+  pair_tiling(p, EPI == GEMM_DW, BN);
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1714,7 +1730,8 @@ int launch_pairs(const CUtensorMap& ta, const CUtensorMap& tb, Params p, cudaStr
   p.tail_kbps = p.num_kb;
   p.part = nullptr;
   if (plan) *plan = TailPlan{0, 0, 0, 0, 0};
-  if ((EPI == GEMM_DW || ((EPI == GEMM_FWD || EPI == GEMM_DX) && p.num_kb >= kTailMinKb)) &&
+  if (BN == 256 &&
+      (EPI == GEMM_DW || ((EPI == GEMM_FWD || EPI == GEMM_DX) && p.num_kb >= kTailMinKb)) &&
       tail_ws && plan && p.splits == 1) {
     const TailPlan tp = tail_plan(p.M, p.N, p.Kred, max_clusters);
     const size_t ctr = EPI == GEMM_DW ? 0 : kTailCtrBytes;
@@ -1848,6 +1865,10 @@ int launch_gemm(const GemmLaunch& g, cudaStream_t stream) {
         }
         return launch_tiles<128, false, false, GEMM_FWD, true>(ta, tb, p, stream);
       }
+      if (g2.pair && pair_bn(g.M, g.N, 1) == 128) {
+        if (!make_map(&tb, g.B, g.Kred, g.N, BK, 64)) return 3;
+        return launch_pairs<false, false, GEMM_FWD, false, false, false, 128>(ta, tb, p, stream);
+      }
       if (!make_map(&tb, g.B, g.Kred, g.N, BK, g2.pair ? 128 : 256)) return 3;
       if (g2.pair) {
         // with a workspace, the last wave's tiles as reduction slices
@@ -1860,11 +1881,17 @@ int launch_gemm(const GemmLaunch& g, cudaStream_t stream) {
       // 2-SM tiles whatever the tiling mode: E4M3 rows of 128 elements
       if (g.a_wrap && (g.a_wrap % 128 != 0 || g.Kred != 2 * g.a_wrap)) return 1;
       if (!make_map(&ta, g.A, g.a_wrap ? g.a_wrap : g.Kred, g.M, 128, BM, 1)) return 3;
+      if (pair_bn(g.M, g.N, 1) == 128) {
+        if (!make_map(&tb, g.B, g.Kred, g.N, 128, 64, 1)) return 3;
+        return launch_pairs<false, false, GEMM_FWD8, false, false, false, 128>(ta, tb, p, stream);
+      }
       if (!make_map(&tb, g.B, g.Kred, g.N, 128, 128, 1)) return 3;
       return launch_pairs<false, false, GEMM_FWD8>(ta, tb, p, stream);
     case GEMM_DX:
       if (!make_map(&ta, g.A, g.Kred, g.M, BK, BM, 2, static_cast<uint64_t>(g.lda))) return 3;
       if (!make_map(&tb, g.B, g.N, g.Kred, 64, BK)) return 3;
+      if (g2.pair && pair_bn(g.M, g.N, 1) == 128)
+        return launch_pairs<false, true, GEMM_DX, false, false, false, 128>(ta, tb, p, stream);
       if (g2.pair) {
         TailPlan tp{0, 0, 0, 0, 0};
         return launch_pairs<false, true, GEMM_DX>(ta, tb, p, stream, g.ws, g.ws_bytes,
@@ -1908,7 +1935,10 @@ int launch_gemm(const GemmLaunch& g, cudaStream_t stream) {
       ps.v = nullptr;
       ps.changed = nullptr;
       ps.dW_out = static_cast<float*>(g.ws);
-      const int rc = launch_pairs<true, true, GEMM_DW>(ta, tb, ps, stream);
+      const int rc =
+          pair_bn(g.M, g.N, p.splits) == 128
+              ? launch_pairs<true, true, GEMM_DW, false, false, false, 128>(ta, tb, ps, stream)
+              : launch_pairs<true, true, GEMM_DW>(ta, tb, ps, stream);
       if (rc) return rc;
       if (!g.W) {
         // gradient only: sum the slabs into dW_out
