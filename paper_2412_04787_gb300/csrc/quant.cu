@@ -9,6 +9,8 @@
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
 
+#include <numeric>
+
 #include "dqt_internal.h"
 
 namespace dqt {
@@ -292,7 +294,9 @@ struct RowRing {
   }
 
   // All lanes of the consumer warp: waits for chunk j; false (warp-uniform,
-  // timeout recorded) if it did not arrive in time.
+  // timeout recorded) if it did not arrive in time.  The warp has taken a row
+  // of the slot's previous chunk itself (ring_geometry), so that chunk's phase
+  // is complete.
   __device__ __forceinline__ bool acquire(int j, int lane, unsigned int* status,
                                           uint64_t limit_ns) const {
     const bool ok = __all_sync(0xffffffffu, mbar_wait(&full[j % S], (j / S) & 1, limit_ns));
@@ -696,17 +700,29 @@ namespace {
 
 // Geometry of a row ring (act_quant_bulk_kernel, codes_to_xdq_bulk_kernel):
 // chunks of about 8 KB (rows of up to 8 KB are copied one per chunk), then as
-// many slots as fit in kAqbRing bytes (48 at most) and up to kRingWarps
-// consumer warps, no more than the rows that the slots hold; false when fewer
-// than four chunks fit.  One producer thread issues a bulk copy about every
-// 0.2 us whatever its size, so copies below ~8 KB leave the ring short of
-// bytes in flight.
-bool ring_geometry(int64_t row_bytes, int& rpc, int& W, int& S) {
+// many slots as fit in kAqbRing bytes (48 at most) and up to max_warps consumer
+// warps; false when fewer than four chunks fit.  One producer thread issues a
+// bulk copy about every 0.2 us whatever its size, so copies below ~8 KB leave
+// the ring short of bytes in flight.
+//
+// S rpc is a multiple of W: the row that a warp waits for and the one that used
+// the same place of the ring before, S rpc rows earlier, are then the same
+// warp's.  A warp that could reach a slot before the slot's previous chunk had
+// landed would wait on a phase parity that reads as complete.
+bool ring_geometry(int64_t row_bytes, int max_warps, int& rpc, int& W, int& S) {
   rpc = row_bytes >= 8192 ? 1 : static_cast<int>(8192 / row_bytes);
-  const int64_t smax = kAqbRing / (rpc * row_bytes);
-  if (smax < 4) return false;
-  S = static_cast<int>(smax < 48 ? smax : 48);
-  W = S * rpc < kRingWarps ? S * rpc : kRingWarps;
+  const int64_t fit = kAqbRing / (rpc * row_bytes);
+  if (fit < 4) return false;
+  const int smax = static_cast<int>(fit < 48 ? fit : 48);
+  S = W = 0;
+  for (int w = max_warps < smax * rpc ? max_warps : smax * rpc; w > 0; --w) {
+    const int unit = w / std::gcd(w, rpc);  // S is a multiple of it
+    const int s = smax / unit * unit;
+    if (w * s > W * S) {
+      W = w;
+      S = s;
+    }
+  }
   return true;
 }
 constexpr int kRingMaxSmem = kAqbRing + 16 * 48 + 512 * kRingWarps;  // ring, barriers, tables
@@ -739,8 +755,7 @@ template <bool F8, bool IMG, int XDQ>
 int launch_aq_ring(const uint16_t* X, int64_t T, int64_t K, int8_t* Xq, float* s_x,
                    uint16_t* Xq_img, uint16_t* Xdq, cudaStream_t stream) {
   int rpc, W, S;
-  if (!ring_geometry(2 * K, rpc, W, S)) return -1;
-  if (XDQ == 2 && W > 16) W = 16;
+  if (!ring_geometry(2 * K, XDQ == 2 ? 16 : kRingWarps, rpc, W, S)) return -1;
   static bool attr_set = false;  // per template instance
   return launch_ring(act_quant_bulk_kernel<F8, IMG, XDQ>, attr_set, XDQ == 2, T, rpc, W, S, 2 * K,
                      stream, X, static_cast<int>(T), static_cast<int>(K), Xq, s_x, Xq_img, Xdq);
@@ -783,7 +798,7 @@ int launch_codes_to_xdq(const int8_t* Xq, const float* s_x, int64_t T, int64_t K
                         cudaStream_t stream) {
   {
     int rpc, W, S;
-    if (ring_geometry(K, rpc, W, S)) {
+    if (ring_geometry(K, kRingWarps, rpc, W, S)) {
       static bool attr_set = false;
       return launch_ring(codes_to_xdq_bulk_kernel, attr_set, false, T, rpc, W, S, K, stream, Xq, s_x,
                          static_cast<int>(T), static_cast<int>(K), Xdq);

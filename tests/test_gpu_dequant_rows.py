@@ -60,3 +60,25 @@ def test_codes_to_xdq_at_extreme_scales(s):
     sx = torch.full((7,), s)
     got = dqt.dqt_codes_to_xdq(q.cuda(), sx.cuda()).cpu()
     assert _same(got, torch.div(q.float(), sx[:, None]).to(torch.bfloat16))
+
+
+@pytest.mark.parametrize("T,K", [(8192, 5632), (16384, 768), (8192, 2048), (8192, 1040), (4096, 4112)])
+def test_row_ring_many_rounds(T, K):
+    """Many rounds of the shared-memory row ring (each slot refilled up to ten
+    times), launched again and again: a warp that took a slot's old rows, or
+    released a slot early, would change bytes or run into a wait's limit."""
+    x = torch.randn(T, K, generator=torch.Generator().manual_seed(K)).to(torch.bfloat16).cuda()
+    first = None
+    for _ in range(60):
+        out = list(dqt.dqt_act_quant_images(x)) + list(dqt.dqt_act_quant_fp8(x))
+        out.append(dqt.dqt_codes_to_xdq(out[0], out[1]))
+        if first is None:
+            first = out
+        else:
+            for a, b in zip(out, first):
+                assert torch.equal(a, b)
+    dqt.dqt_check_device_status()
+    s = 127.0 / x.float().abs().amax(1).double().clamp_min(1e-5)
+    assert torch.equal(first[1], s.float())
+    want = (x.float() * first[1][:, None]).round().clamp_(-128, 127)
+    assert torch.equal(first[0].float(), want)
