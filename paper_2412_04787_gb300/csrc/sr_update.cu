@@ -88,14 +88,16 @@ __device__ __forceinline__ void store_images4(uint16_t* img, uint8_t* img8, int6
 // parameter space); SLABS: the gradient may be split into slabs and the
 // summed gradient written out, and the images of the new codes (img bf16,
 // img8 E4M3, direct or split as in store_e4m3_4; int8 codes only) written
-// beside them.  The plain instance is the leanest stream.
+// beside them.  The plain instance is the leanest stream.  pc: the generator's
+// per-call parts for constants passed by value (23 M weights 86.6 -> 83.6 us).
 template <bool packed, bool DEV, bool SLABS>
 __global__ void __launch_bounds__(kThreads, SLABS ? 4 : 5)
     sr_update_kernel(const float* __restrict__ grad, int nsplit, long long slab,
                      float* __restrict__ g_out, int8_t* __restrict__ W, float* __restrict__ m,
                      float* __restrict__ v, int64_t numel, const UpdateConsts uc_arg,
                      const UpdateConsts* __restrict__ uc_dev, unsigned long long* changed,
-                     uint16_t* __restrict__ img, uint8_t* __restrict__ img8, int64_t img8_k) {
+                     uint16_t* __restrict__ img, uint8_t* __restrict__ img8, int64_t img8_k,
+                     const PhiloxCall pc) {
   dep_wait();
   dep_trigger();
   uint8_t* Wp = reinterpret_cast<uint8_t*>(W);
@@ -114,8 +116,9 @@ __global__ void __launch_bounds__(kThreads, SLABS ? 4 : 5)
     if (SLABS && g_out) __stcs(reinterpret_cast<float4*>(g_out + e), g4);
     uint4 w = make_uint4(0, 0, 0, 0);
     if (uc.round_mode == 0)
-      w = sr_words(global_blk(uc, static_cast<uint64_t>(gi)), uc.step_lo, uc.tensor_id, uc.key0,
-                   uc.key1);
+      w = DEV ? sr_words(global_blk(uc, static_cast<uint64_t>(gi)), uc.step_lo, uc.tensor_id, uc.key0,
+                         uc.key1)
+              : philox_call(global_blk(uc, static_cast<uint64_t>(gi)), pc);
     const int32_t a = dqt_update_elem(uc, g4.x, c4.x, m4.x, v4.x, w.x);
     const int32_t b = dqt_update_elem(uc, g4.y, c4.y, m4.y, v4.y, w.y);
     const int32_t c = dqt_update_elem(uc, g4.z, c4.z, m4.z, v4.z, w.z);
@@ -344,7 +347,7 @@ int sr_launch(const float* grad, int splits, long long slab, float* g_out, int8_
                uint8_t* img8 = nullptr, int64_t img8_k = 0) {
   return launch_dep(sr_update_kernel<packed, DEV, SLABS>, stream_blocks(numel), kThreads, 0, stream,
                     grad, splits, slab, g_out, W, m, v, numel, uc, uc_dev, changed, img, img8,
-                    img8_k);
+                    img8_k, philox_call_consts(uc));
 }
 
 template <bool packed>
