@@ -330,7 +330,7 @@ class MLPStep:
         # kernel launches per step: act_quant 2, weight images 3 (+3 E4M3),
         # forward 3, dX 3, and per projection the dW GEMM, the streaming
         # kernel of its sliced last wave (when the shape has one), and for
-        # Adafactor the five statistics kernels and the step; with int8
+        # Adafactor the three statistics kernels and the step; with int8
         # operands each forward call converts both operands (3 x 2 images
         # instead of the 3 shared weight images), each dX call the weight
         # and each dW call X_tilde (3 + 3)
@@ -359,7 +359,7 @@ class MLPStep:
             self.kinds = (["act_quant_fp8", "codes_to_fp8", "codes_to_bf16", "fwd_fp8"] if fp8 else
                           ["act_quant", "codes_to_bf16", "fwd"]) + ["bwd_dx", self.dw_kind]
         if optimizer == "adafactor":
-            self.launches_per_step += 3 * 6
+            self.launches_per_step += 3 * 4
         if self.nimg:  # no conversion launches: the updates write the images
             self.kinds = [k for k in self.kinds if k not in ("codes_to_bf16", "codes_to_fp8")]
 

@@ -35,22 +35,28 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // One 16-byte vector (four pairs of one head) per thread step.  cs holds
 // (cos, sin) per position and pair: fp32 [S, D/2, 2].  A block takes R whole
 // rows side by side (one when a row has as many vectors as the block has
-// threads, or more), so that the row, the position and the vector in the head
-// cost two 32-bit remainders per thread instead of three 64-bit divisions per
-// vector, and the blocks run through memory in order: 8 x 2048 x 32 x 64 in
-// 23.8 us, 28.9 before (134 MB: 5.6 TB/s).
+// threads, or more) and the blocks run through memory in order: the position
+// is a remainder of block indices, and the vector in the head a mask where a
+// head has a power of two of them (head_mask, else -1). Three 64-bit divisions
+// per vector had bound the kernel; two 32-bit remainders per thread still took
+// half of its instructions. 8 x 2048 x 32 x 64 (134 MB): 28.9 -> 23.8 ->
+// 22.5 us.
 template <bool INV>
 __global__ void __launch_bounds__(kRopeThreads)
     rope_kernel(const uint4* __restrict__ x, uint4* __restrict__ y, const float4* __restrict__ cs,
-                int64_t rows, int row_vecs, uint32_t S, int head_vecs, int R) {
+                int64_t rows, int row_vecs, uint32_t S, int head_vecs, int head_mask,
+                int R) {
   dep_wait();
   const int tr = row_vecs < kRopeThreads ? static_cast<int>(threadIdx.x) / row_vecs : 0;
   const int64_t row = static_cast<int64_t>(blockIdx.x) * R + tr;
   if (tr >= R || row >= rows) return;
-  const float4* table = cs + static_cast<int64_t>(static_cast<uint32_t>(row) % S) * head_vecs * 2;
+  // the position: a remainder of block indices, then tr steps
+  uint32_t pos = (blockIdx.x * static_cast<uint32_t>(R)) % S + static_cast<uint32_t>(tr);
+  if (pos >= S) pos = pos - S < S ? pos - S : pos % S;
+  const float4* table = cs + static_cast<int64_t>(pos) * head_vecs * 2;
   for (int v = static_cast<int>(threadIdx.x) - tr * row_vecs; v < row_vecs; v += kRopeThreads) {
     // four pairs = eight floats = two float4 of the table
-    const float4* t = table + 2 * (v % head_vecs);
+    const float4* t = table + 2 * (head_mask >= 0 ? v & head_mask : v % head_vecs);
     const uint4 xv = __ldcs(x + row * row_vecs + v);
     const float4 c01 = __ldg(t), c23 = __ldg(t + 1);
     const float cth[4] = {c01.x, c01.z, c23.x, c23.z};
@@ -338,7 +344,9 @@ __global__ void __launch_bounds__(32 * kNormWarps)
 // it reads itself), and keeps its dw partial sums in registers; at the end the
 // block's groups add theirs in order in shared memory and write one partial
 // row part[block, :] (fp32): an eighth of the bytes that a row per warp took
-// for the column pass.  16384 x 2048: 58.4 -> 46 us with that pass.
+// for the column pass.  The gain sits in shared memory (from L1, with nothing
+// to spare in registers, its reads were what the warps waited for).  16384 x
+// 2048, with the column pass: 58.4 -> 46 -> 36.6 us.
 constexpr int kNormBwdWarps = 16;
 constexpr int kNormStages = 3;
 template <int VPL>
@@ -364,6 +372,7 @@ __global__ void __launch_bounds__(32 * kNormBwdWarps, 1)
   constexpr int G = kNormBwdWarps / WPR;       // row groups per block
   __shared__ float4 sums[VPL * WPR * 64];      // one row of columns
   __shared__ float dots[2][G][WPR];            // the warps' parts of a row's sum, two rows in turn
+  __shared__ uint4 gain[VPL * WPR * 32];       // w, read twice per row
   extern __shared__ uint4 norm_ring[];         // [warp][stage][x, dy][VPL * 32]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int grp = warp / WPR, sub = warp % WPR;
@@ -372,8 +381,8 @@ __global__ void __launch_bounds__(32 * kNormBwdWarps, 1)
   const float inv_d = 1.0f / static_cast<float>(nv * 8);
   uint4* ring = norm_ring + warp * (kNormStages * 2 * VPL * 32);
   const int c0 = sub * 32 + lane;  // vector k of this lane: column c0 + 32 WPR k
-  // the gain vector is re-read per row from L1 (it is D * 2 bytes) rather
-  // than held in registers next to the partial sums
+  for (int i = threadIdx.x; i < nv; i += 32 * kNormBwdWarps) gain[i] = __ldg(w + i);
+  __syncthreads();
   float acc[VPL][8];
 #pragma unroll
   for (int k = 0; k < VPL; ++k)
@@ -409,7 +418,7 @@ __global__ void __launch_bounds__(32 * kNormBwdWarps, 1)
     for (int k = 0; k < VPL; ++k) {
       const int c = c0 + 32 * WPR * k;
       if (c >= nv) break;
-      const uint4 wv = __ldg(w + c), xv = xs[32 * k], gv = gs[32 * k];
+      const uint4 wv = gain[c], xv = xs[32 * k], gv = gs[32 * k];
       const uint32_t a[4] = {xv.x, xv.y, xv.z, xv.w};
       const uint32_t g[4] = {gv.x, gv.y, gv.z, gv.w};
       const uint32_t b[4] = {wv.x, wv.y, wv.z, wv.w};
@@ -436,7 +445,7 @@ __global__ void __launch_bounds__(32 * kNormBwdWarps, 1)
     for (int k = 0; k < VPL; ++k) {
       const int c = c0 + 32 * WPR * k;
       if (c >= nv) break;
-      const uint4 wv = __ldg(w + c), xv = xs[32 * k], gv = gs[32 * k];
+      const uint4 wv = gain[c], xv = xs[32 * k], gv = gs[32 * k];
       const uint32_t a[4] = {xv.x, xv.y, xv.z, xv.w};
       const uint32_t g[4] = {gv.x, gv.y, gv.z, gv.w};
       const uint32_t b[4] = {wv.x, wv.y, wv.z, wv.w};
@@ -530,7 +539,8 @@ int launch_rope(const uint16_t* x, uint16_t* y, const float* cos_sin, int64_t ro
   auto* yv = reinterpret_cast<uint4*>(y);
   auto* cv = reinterpret_cast<const float4*>(cos_sin);
   return launch_dep(inverse ? rope_kernel<true> : rope_kernel<false>, blocks, kRopeThreads, 0,
-                    stream, xv, yv, cv, rows, row_vecs, static_cast<uint32_t>(S), head_vecs, R);
+                    stream, xv, yv, cv, rows, row_vecs, static_cast<uint32_t>(S), head_vecs,
+                    (head_vecs & (head_vecs - 1)) == 0 ? head_vecs - 1 : -1, R);
 }
 
 int launch_ce_fwd(const uint16_t* logits, const int64_t* targets, int64_t M, int64_t V,
