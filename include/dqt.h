@@ -220,9 +220,10 @@ int dqt_bitlinear_fwd(const int8_t* Xq, const float* s_x, const int8_t* W, float
  * ws: NULL, or a device workspace of at least dqt_fwd_img_workspace_size(T, K,
  * N) bytes (16-byte aligned; DQT_ERR_ARG if smaller).  With it, when the
  * output's 256 x 256 tiles leave the last wave of the 2-SM kernel short, the
- * tiles of that wave are cut into reduction slices whose fp32 partials go to
- * the workspace, and the last slice to finish a region adds them in slice
- * order and applies the epilogue; every partial is an exact integer, so Y and
+ * tiles of that wave are cut into reduction slices whose partials (fp32;
+ * int32 where the grid needs a chunked accumulation) go to the workspace, and
+ * the last slice to finish a region adds them in slice order and applies the
+ * epilogue; every partial is an exact integer, so Y and
  * acc are those of the uncut kernel bit for bit.  The size is 0 (any ws) when
  * no cut is planned.  A workspace serves one call at a time. */
 size_t dqt_fwd_img_workspace_size(int64_t T, int64_t K, int64_t N);
