@@ -6,7 +6,7 @@
 // codes.  Four launches, each HBM-bound or tiny:
 //
 //   af_sq_partials  one read of G (and the codes): per 128-column chunk row
-//                   sums and per 32-row slab column sums of g^2 + eps1, and the
+//                   sums and per row slab column sums of g^2 + eps1, and the
 //                   sum of c^2 (for the parameter RMS), in a fixed order
 //   af_moments      R <- b2 R + (1 - b2) mean_k, C <- b2 C + (1 - b2) mean_n,
 //                   and (the last row block to finish) Rbar = mean R
@@ -30,7 +30,7 @@ namespace dqt {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kRowsPerSlab = 32;           // rows per af_sq/usq block
+constexpr int kRowsPerSlab = 32;           // most rows per af_sq/usq block (slab_rows)
 constexpr int kColsPerBlock = kThreads * 4;  // 1024 columns per block (float4 per thread)
 
 __device__ __forceinline__ char4 load_codes4(const int8_t* W, bool packed, int64_t e) {
@@ -59,14 +59,15 @@ constexpr int kUnroll = 4;
 
 __global__ void __launch_bounds__(kThreads, 4)
     af_sq_partials_kernel(const float* __restrict__ G, const int8_t* __restrict__ W, bool packed,
-                          bool need_csq, int N, int K, float eps1, float* __restrict__ rowpart,
-                          float* __restrict__ colpart, unsigned long long* __restrict__ cpart,
+                          bool need_csq, int N, int K, int rows, float eps1,
+                          float* __restrict__ rowpart, float* __restrict__ colpart,
+                          unsigned long long* __restrict__ cpart,
                           unsigned int* __restrict__ done) {
   dep_wait();
   __shared__ unsigned long long sh[kThreads / 32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int k0 = blockIdx.x * kColsPerBlock + threadIdx.x * 4;
-  const int n0 = blockIdx.y * kRowsPerSlab;
+  const int n0 = blockIdx.y * rows;
   const bool col_ok = k0 < K;  // K is a multiple of 4: the whole float4 is in range
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2)
     done[threadIdx.x] = 0;  // the counts of finished blocks of the two kernels that follow
@@ -74,7 +75,7 @@ __global__ void __launch_bounds__(kThreads, 4)
   uint32_t csq = 0;  // at most 32 rows x 4 codes x 128^2 per thread
   const int chunk = blockIdx.x * (kColsPerBlock / 128) + warp;  // this warp's 128-column chunk
   const int nchunks = (K + 127) / 128;
-  for (int r0 = 0; r0 < kRowsPerSlab && n0 + r0 < N; r0 += kUnroll) {
+  for (int r0 = 0; r0 < rows && n0 + r0 < N; r0 += kUnroll) {
     float4 g[kUnroll];
     char4 c[kUnroll];
 #pragma unroll
@@ -126,7 +127,7 @@ __global__ void __launch_bounds__(kThreads, 4)
 // The first row_blocks blocks finish the row means (one thread per row, its
 // 128-column chunk partials in order); the others the column means: 32
 // columns per block, eight threads per column each summing every eighth
-// 32-row slab partial, then the eight sums combined in order in shared memory.
+// row slab's partial, then the eight sums combined in order in shared memory.
 __global__ void __launch_bounds__(kThreads)
     af_moments_kernel(const float* __restrict__ rowpart, const float* __restrict__ colpart,
                       int nchunks, int nslabs, int N, int K, int row_blocks, float b2, float omb2,
@@ -169,7 +170,8 @@ __global__ void __launch_bounds__(kThreads)
   float s0 = 0.f, s1 = 0.f;
   if (k < K) {
     int j = ty;
-    for (; j + 8 < nslabs; j += 16) {  // two loads in flight per thread
+#pragma unroll 4
+    for (; j + 8 < nslabs; j += 16) {  // eight loads in flight per thread
       s0 += colpart[static_cast<int64_t>(j) * K + k];
       s1 += colpart[static_cast<int64_t>(j + 8) * K + k];
     }
@@ -190,6 +192,11 @@ __device__ __forceinline__ float af_u(float g, float an, float bk) {
   return __fmul_rn(__fmul_rn(g, an), bk);
 }
 
+__device__ __forceinline__ float4 load_row(const float* col, int r, int K, bool ok) {
+  return ok ? __ldcs(reinterpret_cast<const float4*>(col + static_cast<int64_t>(r) * K))
+            : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 // The factors a[n] = 1 / sqrt(R[n] / Rbar) and b[k] = 1 / sqrt(C[k]) of this
 // block's rows and columns, each from correctly rounded fp32 operations (the
 // first block of a row or column range writes them out), and the block's sum
@@ -198,6 +205,8 @@ __device__ __forceinline__ float af_u(float g, float an, float bk) {
 // decay, rms_u, rms_x, alpha}.  Factors and scalars had launches of their own,
 // 6.7 and 6.9 us of latency for a few thousand values (the statistics of 5632 x
 // 2048, replayed: 40.2 -> 38.0 us).
+// The first rows are loaded before the factors are formed, and the parameter
+// RMS, fp64 on one thread, is formed only where it is used: 27.8 -> 25.0 us.
 struct FinalArgs {
   float s_w, rho, eps2, clip_d, weight_decay;
   int scale_parameter;
@@ -205,8 +214,9 @@ struct FinalArgs {
 
 __global__ void __launch_bounds__(kThreads)
     af_usq_kernel(const float* __restrict__ G, const float* __restrict__ R,
-                  const float* __restrict__ C, int N, int K, float* __restrict__ a, float* __restrict__ b,
-                  float* __restrict__ upart, const unsigned long long* __restrict__ cpart,
+                  const float* __restrict__ C, int N, int K, int rows,
+                  float* __restrict__ a, float* __restrict__ b, float* __restrict__ upart,
+                  const unsigned long long* __restrict__ cpart,
                   unsigned int* __restrict__ done, const FinalArgs h, float* out) {
   dep_wait();
   __shared__ float sh[kThreads / 32];
@@ -215,8 +225,13 @@ __global__ void __launch_bounds__(kThreads)
   __shared__ float an_s[kRowsPerSlab];
   __shared__ bool last_s;
   const int k0 = blockIdx.x * kColsPerBlock + threadIdx.x * 4;
-  const int n0 = blockIdx.y * kRowsPerSlab;
-  if (threadIdx.x < kRowsPerSlab && n0 + static_cast<int>(threadIdx.x) < N) {
+  const int n0 = blockIdx.y * rows;
+  // the first rows' loads are on their way while the factors are formed
+  const float* col = G + static_cast<int64_t>(n0) * K + k0;
+  float4 g[kUnroll];
+#pragma unroll
+  for (int u = 0; u < kUnroll; ++u) g[u] = load_row(col, u, K, k0 < K && u < rows && n0 + u < N);
+  if (static_cast<int>(threadIdx.x) < rows && n0 + static_cast<int>(threadIdx.x) < N) {
     const int n = n0 + threadIdx.x;
     const float an = __fdiv_rn(1.0f, __fsqrt_rn(__fdiv_rn(R[n], out[0])));
     an_s[threadIdx.x] = an;
@@ -230,14 +245,10 @@ __global__ void __launch_bounds__(kThreads)
         __fdiv_rn(1.0f, __fsqrt_rn(c4.x)), __fdiv_rn(1.0f, __fsqrt_rn(c4.y)),
         __fdiv_rn(1.0f, __fsqrt_rn(c4.z)), __fdiv_rn(1.0f, __fsqrt_rn(c4.w)));
     if (blockIdx.y == 0) *reinterpret_cast<float4*>(b + k0) = bk;
-    for (int r0 = 0; r0 < kRowsPerSlab && n0 + r0 < N; r0 += kUnroll) {
-      float4 g[kUnroll];
+    for (int r0 = 0; r0 < rows && n0 + r0 < N; r0 += kUnroll) {
+      if (r0)
 #pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        const int n = n0 + r0 + u;
-        g[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (n < N) g[u] = __ldcs(reinterpret_cast<const float4*>(G + static_cast<int64_t>(n) * K + k0));
-      }
+        for (int u = 0; u < kUnroll; ++u) g[u] = load_row(col, r0 + u, K, n0 + r0 + u < N);
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
         if (n0 + r0 + u >= N) break;
@@ -263,14 +274,16 @@ __global__ void __launch_bounds__(kThreads)
 #pragma unroll 4
   for (int i = threadIdx.x; i < nparts; i += kThreads) {
     us += static_cast<double>(__ldcg(upart + i));
-    cs += cpart[i];
+    if (h.scale_parameter) cs += cpart[i];
   }
   us = block_sum(us, shd);
-  cs = block_sum(cs, shu);
+  if (h.scale_parameter) cs = block_sum(cs, shu);
   if (threadIdx.x == 0) {
     const double nk = static_cast<double>(N) * static_cast<double>(K);
     const double rms_u = sqrt(us / nk);
-    const double rms_x = sqrt(static_cast<double>(cs) / nk) / static_cast<double>(h.s_w);
+    // without parameter scaling the codes were not read, and rms_x is 0
+    const double rms_x = h.scale_parameter
+        ? sqrt(static_cast<double>(cs) / nk) / static_cast<double>(h.s_w) : 0.0;
     const double alpha = static_cast<double>(h.rho) *
                          (h.scale_parameter ? fmax(static_cast<double>(h.eps2), rms_x) : 1.0);
     const double div = fmax(1.0, rms_u / static_cast<double>(h.clip_d));
@@ -346,8 +359,21 @@ __global__ void __launch_bounds__(kThreads)
   if (changed) add_changed(changed, n_changed);
 }
 
+// Rows per block of the two passes over the gradient: halved while the grid
+// is below two blocks per SM (152), each block then having fewer rounds of
+// loads to wait for (statistics of 2048 x 768: 22.5 -> 17.0 us, of 512 x 512:
+// 20.6 -> 15.7; where 32 rows give more blocks, 16 are no faster: 27.6 against
+// 28.0 us at 5632 x 2048, 32.1 against 30.9 at 2048 x 5632).  The column sums'
+// chains keep their length (rows in a block plus blocks per sum), their error
+// against 64 bits is 5.8e-8 rms either way.
+int slab_rows(int64_t N, int64_t gx) {
+  int rows = kRowsPerSlab;
+  while (rows > 8 && gx * ((N + rows - 1) / rows) < 304) rows >>= 1;
+  return rows;
+}
+
 struct Layout {
-  int nchunks, nslabs, gx, nparts;
+  int nchunks, nslabs, gx, nparts, rows;
   size_t row_off, col_off, cpart_off, upart_off, scal_off, a_off, b_off, rsum_off, done_off, bytes;
 };
 
@@ -356,8 +382,9 @@ size_t align256(size_t x) { return (x + 255) & ~static_cast<size_t>(255); }
 Layout layout(int64_t N, int64_t K) {
   Layout L{};
   L.nchunks = static_cast<int>((K + 127) / 128);
-  L.nslabs = static_cast<int>((N + kRowsPerSlab - 1) / kRowsPerSlab);
   L.gx = static_cast<int>((K + kColsPerBlock - 1) / kColsPerBlock);
+  L.rows = slab_rows(N, L.gx);
+  L.nslabs = static_cast<int>((N + L.rows - 1) / L.rows);
   L.nparts = L.gx * L.nslabs;
   L.row_off = 0;
   L.col_off = align256(L.row_off + static_cast<size_t>(L.nchunks) * N * 4);
@@ -400,7 +427,7 @@ int launch_adafactor_stats(const float* G, const int8_t* W, bool packed, float s
   unsigned int* done = reinterpret_cast<unsigned int*>(base + L.done_off);
   const dim3 grid(L.gx, L.nslabs);
   if (launch_dep(af_sq_partials_kernel, grid, kThreads, 0, stream, G, W, packed,
-                 h.scale_parameter != 0, n, k, h.eps1, rowpart, colpart, cpart, done))
+                 h.scale_parameter != 0, n, k, L.rows, h.eps1, rowpart, colpart, cpart, done))
     return 3;
   const int row_blocks = (n + kThreads - 1) / kThreads;
   const int col_blocks = (k + 31) / 32;
@@ -409,7 +436,7 @@ int launch_adafactor_stats(const float* G, const int8_t* W, bool packed, float s
                  scalars_out))
     return 3;
   const FinalArgs fa = {s_w, h.rho, h.eps2, h.clip_d, h.weight_decay, h.scale_parameter};
-  return launch_dep(af_usq_kernel, grid, kThreads, 0, stream, G, R, C, n, k, a_out, b_out, upart,
+  return launch_dep(af_usq_kernel, grid, kThreads, 0, stream, G, R, C, n, k, L.rows, a_out, b_out, upart,
                     cpart, done + 1, fa, scalars_out);
 }
 
