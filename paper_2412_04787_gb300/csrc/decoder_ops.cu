@@ -112,15 +112,21 @@ __device__ __forceinline__ float ex2(float t) {
 }
 
 // One block per row; V a multiple of 8 (16-byte vectors of bf16).  A thread
-// takes kCeVecs vectors at a time, their loads in flight together: the
+// takes VECS vectors at a time, their loads in flight together: the
 // chunk's maximum on bf16 pairs (exact; a NaN makes the row's sum NaN), one
 // rescaling of the running sum, then exp(x - max) as 2^((x - max) log2 e),
 // the difference formed before the product, so the product's rounding is
 // 2^-24 of an exponent that is small wherever the term counts.  With expf
 // and a maximum and rescaling per vector the kernel was bound by instruction
 // issue: 8192 x 32000 rows, forward and gradient together, 286 -> 244 us.
-constexpr int kCeVecs = 8;
+// VECS is the least that takes the row in ceil(V / 16384) steps, since a
+// thread forms VECS * 8 exponentials whether its vectors lie in the row or
+// not: 8192 rows of 1000, 4096, 10000, 18000 and 32000, forward alone, 17.2,
+// 24.8, 36.8, 55.7 and 80.9 us; eight vectors throughout 31.7, 44.8, 47.2, 71.6
+// and 81.0; expf with two vectors in flight 20.6, 32.7, 55.5, 82.3 and 129.4.
+constexpr int kCeMaxVecs = 8;
 
+template <int VECS>
 __global__ void __launch_bounds__(kCeThreads)
     ce_fwd_kernel(const uint4* __restrict__ logits, const int64_t* __restrict__ tgt, int64_t V,
                   float* __restrict__ lse, float* __restrict__ row_loss) {
@@ -131,17 +137,17 @@ __global__ void __launch_bounds__(kCeThreads)
   const int nv = static_cast<int>(V >> 3);
   const uint4* row = logits + r * nv;
   float m = -INFINITY, s = 0.0f;
-  for (int i0 = threadIdx.x; i0 < nv; i0 += kCeVecs * kCeThreads) {
-    uint4 v[kCeVecs];
+  for (int i0 = threadIdx.x; i0 < nv; i0 += VECS * kCeThreads) {
+    uint4 v[VECS];
 #pragma unroll
-    for (int k = 0; k < kCeVecs; ++k) {
+    for (int k = 0; k < VECS; ++k) {
       const int i = i0 + k * kCeThreads;
       // past the row: -inf, which adds nothing
       v[k] = i < nv ? __ldcs(row + i) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
     }
     __nv_bfloat162 mx = *reinterpret_cast<const __nv_bfloat162*>(&v[0].x);
 #pragma unroll
-    for (int k = 0; k < kCeVecs; ++k) {
+    for (int k = 0; k < VECS; ++k) {
       const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) mx = __hmax2_nan(mx, *reinterpret_cast<const __nv_bfloat162*>(&w[j]));
@@ -156,7 +162,7 @@ __global__ void __launch_bounds__(kCeThreads)
     const float mn = fmaxf(m, cm);
     float t0 = 0.0f, t1 = 0.0f;  // two chains
 #pragma unroll
-    for (int k = 0; k < kCeVecs; ++k) {
+    for (int k = 0; k < VECS; ++k) {
       const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -545,8 +551,13 @@ int launch_rope(const uint16_t* x, uint16_t* y, const float* cos_sin, int64_t ro
 
 int launch_ce_fwd(const uint16_t* logits, const int64_t* targets, int64_t M, int64_t V,
                   float* lse, float* row_loss, cudaStream_t stream) {
-  return launch_dep(ce_fwd_kernel, static_cast<unsigned>(M), kCeThreads, 0, stream,
-                    reinterpret_cast<const uint4*>(logits), targets, V, lse, row_loss);
+  const int64_t nv = V >> 3, step = kCeMaxVecs * kCeThreads;
+  const int64_t per_step = (nv + step - 1) / step * kCeThreads;  // threads over all steps
+  decltype(&ce_fwd_kernel<1>) kern[kCeMaxVecs] = {
+      ce_fwd_kernel<1>, ce_fwd_kernel<2>, ce_fwd_kernel<3>, ce_fwd_kernel<4>,
+      ce_fwd_kernel<5>, ce_fwd_kernel<6>, ce_fwd_kernel<7>, ce_fwd_kernel<8>};
+  return launch_dep(kern[(nv + per_step - 1) / per_step - 1], static_cast<unsigned>(M), kCeThreads,
+                    0, stream, reinterpret_cast<const uint4*>(logits), targets, V, lse, row_loss);
 }
 
 int launch_ce_bwd(const uint16_t* logits, const int64_t* targets, const float* lse,
