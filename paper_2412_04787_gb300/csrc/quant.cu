@@ -316,9 +316,11 @@ struct RowRing {
 
 //
 // IMG: the bf16 code image is written; XDQ: the dequantised image, 1 by
-// dq_pair, 2 (long E4M3 rows) from a 256-entry table per row, where the
-// conversions of every element back from E4M3 cost more than the table's
-// (8192 x 5632: 44.2 us by dq_pair, 39.6 from the table; 2048: 13.2 and 14.6).
+// dq_pair, 2 (E4M3 rows beyond 2048) from a 256-entry table per row, where
+// the conversions of every element back from E4M3 cost more than the table's
+// (by dq_pair and from the table, us: 4096 x 1040 6.6 and 8.2, x 2048 8.8 and
+// 9.4, x 4096 15.7 and 12.9, x 5632 22.2 and 17.4; 64 x 4096 6.7 and 4.6, a
+// latency).  Conversions in bit operations on the bytes: 64 x 4096 7.4.
 template <bool F8, bool IMG, int XDQ>
 __global__ void __launch_bounds__(32 * (kRingWarps + 1), 1)
     act_quant_bulk_kernel(const uint16_t* __restrict__ X, int T, int K,
@@ -755,7 +757,7 @@ template <bool F8, bool IMG, int XDQ>
 int launch_aq_ring(const uint16_t* X, int64_t T, int64_t K, int8_t* Xq, float* s_x,
                    uint16_t* Xq_img, uint16_t* Xdq, cudaStream_t stream) {
   int rpc, W, S;
-  if (!ring_geometry(2 * K, XDQ == 2 ? 16 : kRingWarps, rpc, W, S)) return -1;
+  if (!ring_geometry(2 * K, kRingWarps, rpc, W, S)) return -1;
   static bool attr_set = false;  // per template instance
   return launch_ring(act_quant_bulk_kernel<F8, IMG, XDQ>, attr_set, XDQ == 2, T, rpc, W, S, 2 * K,
                      stream, X, static_cast<int>(T), static_cast<int>(K), Xq, s_x, Xq_img, Xdq);
@@ -766,7 +768,8 @@ int launch_aq_bulk(const uint16_t* X, int64_t T, int64_t K, int8_t* Xq, float* s
                    uint16_t* Xq_img, uint16_t* Xdq, cudaStream_t stream) {
   if (F8) {  // (no code image)
     auto launch = !Xdq ? launch_aq_ring<F8, false, 0>
-                       : K > 4096 ? launch_aq_ring<F8, false, F8 ? 2 : 1> : launch_aq_ring<F8, false, 1>;
+                       : K > 2048 ? launch_aq_ring<F8, false, F8 ? 2 : 1>
+                                : launch_aq_ring<F8, false, 1>;
     return launch(X, T, K, Xq, s_x, Xq_img, Xdq, stream);
   }
   auto launch = Xq_img ? (Xdq ? launch_aq_ring<F8, !F8, 1> : launch_aq_ring<F8, !F8, 0>)

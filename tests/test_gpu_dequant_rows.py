@@ -31,6 +31,7 @@ def _same(a, b):
 
 
 @pytest.mark.parametrize("T,K", [(1, 16), (151, 768), (153, 16), (3001, 1040), (20000, 48), (307, 5632),
+                                 (457, 2048), (457, 2064), (700, 4096),
                                  (160, 24576), (5, 49152)])
 def test_xdq_is_the_correctly_rounded_quotient(T, K):
     g = torch.Generator().manual_seed(T + K)
@@ -62,7 +63,8 @@ def test_codes_to_xdq_at_extreme_scales(s):
     assert _same(got, torch.div(q.float(), sx[:, None]).to(torch.bfloat16))
 
 
-@pytest.mark.parametrize("T,K", [(8192, 5632), (16384, 768), (8192, 2048), (8192, 1040), (4096, 4112)])
+@pytest.mark.parametrize("T,K", [(8192, 5632), (16384, 768), (8192, 2048), (8192, 1040), (4096, 4112), (8192, 4096),
+                                 (8192, 3584)])
 def test_row_ring_many_rounds(T, K):
     """Many rounds of the shared-memory row ring (each slot refilled up to ten
     times), launched again and again: a warp that took a slot's old rows, or
