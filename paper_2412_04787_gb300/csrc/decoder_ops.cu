@@ -104,27 +104,19 @@ __device__ __forceinline__ void lse_block(float& m, float& s, float* sh_m, float
   }
 }
 
-// 2^t (the PTX instruction: relative error at most 2^-22).
-__device__ __forceinline__ float ex2(float t) {
-  float r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(t));
-  return r;
-}
-
 // One block per row; V a multiple of 8 (16-byte vectors of bf16).  A thread
-// takes VECS vectors at a time, their loads in flight together: the
-// chunk's maximum on bf16 pairs (exact; a NaN makes the row's sum NaN), one
-// rescaling of the running sum, then exp(x - max) as 2^((x - max) log2 e),
-// the difference formed before the product, so the product's rounding is
-// 2^-24 of an exponent that is small wherever the term counts.  With expf
-// and a maximum and rescaling per vector the kernel was bound by instruction
-// issue: 8192 x 32000 rows, forward and gradient together, 286 -> 244 us.
-// VECS is the least that takes the row in ceil(V / 16384) steps, since a
-// thread forms VECS * 8 exponentials whether its vectors lie in the row or
-// not: 8192 rows of 1000, 4096, 10000, 18000 and 32000, forward alone, 17.2,
-// 24.8, 36.8, 55.7 and 80.9 us; eight vectors throughout 31.7, 44.8, 47.2, 71.6
-// and 81.0; expf with two vectors in flight 20.6, 32.7, 55.5, 82.3 and 129.4.
-constexpr int kCeMaxVecs = 8;
+// takes VECS vectors at a time, their loads in flight together; each vector's
+// maximum (on bf16 pairs, exact) and sum of exp(x - max) join the running pair
+// in order, without the divergent branches of lse_merge (both sides of which
+// a warp walked: two exponentials for one).  Bound by instruction issue, most
+// of it expf.  VECS is the least that takes the row in ceil(V / 12288) steps:
+// 8192 rows of 1000, 4096, 10000, 18000 and 32000, forward alone, 17.4, 29.5,
+// 47.8, 72.8 and 115.3 us; two vectors at a time and branches 20.6, 32.7, 55.5,
+// 82.3 and 129.4; four vectors at most 117.6 and eight 122.5 at 32000.  With 2^t
+// (ex2) for expf and one maximum per step 81 us, but a last bit of lse that
+// differs moves bf16 gradients, and with them 5 % of a decoder's 8-bit codes
+// after three steps, so the arithmetic stays.
+constexpr int kCeMaxVecs = 6;
 
 template <int VECS>
 __global__ void __launch_bounds__(kCeThreads)
@@ -132,7 +124,6 @@ __global__ void __launch_bounds__(kCeThreads)
                   float* __restrict__ lse, float* __restrict__ row_loss) {
   dep_wait();
   __shared__ float sh_m[kCeThreads / 32], sh_s[kCeThreads / 32];
-  constexpr float kLog2e = 1.44269504088896340736f;
   const int64_t r = blockIdx.x;
   const int nv = static_cast<int>(V >> 3);
   const uint4* row = logits + r * nv;
@@ -140,38 +131,28 @@ __global__ void __launch_bounds__(kCeThreads)
   for (int i0 = threadIdx.x; i0 < nv; i0 += VECS * kCeThreads) {
     uint4 v[VECS];
 #pragma unroll
-    for (int k = 0; k < VECS; ++k) {
-      const int i = i0 + k * kCeThreads;
-      // past the row: -inf, which adds nothing
-      v[k] = i < nv ? __ldcs(row + i) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
-    }
-    __nv_bfloat162 mx = *reinterpret_cast<const __nv_bfloat162*>(&v[0].x);
+    for (int k = 0; k < VECS; ++k)
+      if (i0 + k * kCeThreads < nv) v[k] = __ldcs(row + i0 + k * kCeThreads);
 #pragma unroll
     for (int k = 0; k < VECS; ++k) {
+      if (i0 + k * kCeThreads >= nv) break;
       const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+      __nv_bfloat162 mx = *reinterpret_cast<const __nv_bfloat162*>(&w[0]);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) mx = __hmax2_nan(mx, *reinterpret_cast<const __nv_bfloat162*>(&w[j]));
-    }
-    const float lo = __low2float(mx), hi = __high2float(mx), cm = fmaxf(lo, hi);
-    if (cm == -INFINITY && lo == hi) continue;  // nothing but -inf
-    if (lo != lo || hi != hi) {
-      s = lo + hi;
-      m = fmaxf(m, -3.4e38f);  // finite: the merge below drops sums at -inf
-      continue;
-    }
-    const float mn = fmaxf(m, cm);
-    float t0 = 0.0f, t1 = 0.0f;  // two chains
-#pragma unroll
-    for (int k = 0; k < VECS; ++k) {
-      const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+      for (int j = 1; j < 4; ++j) mx = __hmax2(mx, *reinterpret_cast<const __nv_bfloat162*>(&w[j]));
+      const float mv = fmaxf(__low2float(mx), __high2float(mx));
+      float sv = 0.0f;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        t0 += ex2(__fmul_rn(bf16_lo(w[j]) - mn, kLog2e));
-        t1 += ex2(__fmul_rn(bf16_hi(w[j]) - mn, kLog2e));
+        sv += expf(bf16_lo(w[j]) - mv);
+        sv += expf(bf16_hi(w[j]) - mv);
       }
+      const bool up = mv > m;
+      const float e = expf(up ? m - mv : mv - m);
+      const float t = __fmaf_rn(up ? s : sv, e, up ? sv : s);
+      s = mv != -INFINITY ? t : s;
+      m = up ? mv : m;
     }
-    s = s * expf(m - mn) + (t0 + t1);  // the first time 0 * expf(-inf)
-    m = mn;
   }
   lse_block(m, s, sh_m, sh_s);
   if (threadIdx.x == 0) {
@@ -555,7 +536,7 @@ int launch_ce_fwd(const uint16_t* logits, const int64_t* targets, int64_t M, int
   const int64_t per_step = (nv + step - 1) / step * kCeThreads;  // threads over all steps
   decltype(&ce_fwd_kernel<1>) kern[kCeMaxVecs] = {
       ce_fwd_kernel<1>, ce_fwd_kernel<2>, ce_fwd_kernel<3>, ce_fwd_kernel<4>,
-      ce_fwd_kernel<5>, ce_fwd_kernel<6>, ce_fwd_kernel<7>, ce_fwd_kernel<8>};
+      ce_fwd_kernel<5>, ce_fwd_kernel<6>};
   return launch_dep(kern[(nv + per_step - 1) / per_step - 1], static_cast<unsigned>(M), kCeThreads,
                     0, stream, reinterpret_cast<const uint4*>(logits), targets, V, lse, row_loss);
 }
