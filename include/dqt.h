@@ -225,7 +225,10 @@ int dqt_bitlinear_fwd(const int8_t* Xq, const float* s_x, const int8_t* W, float
  * the last slice to finish a region adds them in slice order and applies the
  * epilogue; every partial is an exact integer, so Y and
  * acc are those of the uncut kernel bit for bit.  The size is 0 (any ws) when
- * no cut is planned.  A workspace serves one call at a time. */
+ * no cut is planned.  A workspace serves one call at a time.  Its slice
+ * counters are back at zero when the call has run, so a captured call can be
+ * replayed; after DQT_ERR_TIMEOUT, zero the workspace before the next replay
+ * on it. */
 size_t dqt_fwd_img_workspace_size(int64_t T, int64_t K, int64_t N);
 int dqt_bitlinear_fwd_img(const dqt_bf16* Xq_img, const float* s_x, const dqt_bf16* W_img,
                           float s_w, dqt_grid_t grid, int64_t T, int64_t K, int64_t N,

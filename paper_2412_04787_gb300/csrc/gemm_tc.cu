@@ -95,8 +95,10 @@ struct Params {
   float* part;
   // forward / dX tail: the slices of a tile region are added by the last of
   // them to finish, found with one counter per (tail tile, CTA rank,
-  // epilogue warp): (tag << 16) | slices done, tag unique per launch, so a
-  // counter left by an earlier launch counts as zero
+  // epilogue warp): (tag << 16) | slices done.  The last slice sets it back
+  // to zero, so a replayed launch, whose tag is that of its capture, starts
+  // from zero; the tag makes foreign memory (a workspace's first use) read as
+  // zero too
   unsigned long long* tail_ctr;
   unsigned long long tail_tag;
   // two weights stacked in one call (e.g. a LLaMA MLP's gate and up
@@ -952,6 +954,10 @@ __device__ __forceinline__ bool tail_last(const Params& q, int jt, int rank, int
       assumed = prev;
     }
     done = nv & 0xFFFFull;
+    // every slice has counted: nobody reads the counter again in this launch,
+    // and a replay of a captured launch, which has this launch's tag, counts
+    // from the beginning
+    if (done == static_cast<unsigned long long>(q.tail_splits)) *ctr = 0ull;
   }
   done = __shfl_sync(0xffffffffu, done, 0);
   if (done != static_cast<unsigned long long>(q.tail_splits)) return false;
