@@ -336,7 +336,8 @@ int dqt_bitlinear_bwd_dw_update_img(const dqt_bf16* dY, const dqt_bf16* Xdq, int
  * the slices in slice order and applies the update (bit-identical to
  * dqt_sr_update on that summed gradient).  0 = neither applies to this shape
  * on the current device (or under dqt_set_gemm_tiles(1)).  Passing ws = NULL,
- * or fewer bytes, always runs the single fused kernel.  Slicing gives the same
+ * or fewer bytes, always runs the single fused kernel.  A call without an
+ * update (dW_out only) has no use for a single slice's N K floats.  Slicing gives the same
  * update up to the fp32 summation order of the gradient; it is deterministic
  * for a given shape and device. */
 size_t dqt_bwd_dw_img_workspace_size(int64_t T, int64_t N, int64_t K);

@@ -557,10 +557,14 @@ size_t dqt_bwd_dw_workspace_size(int64_t T, int64_t N, int64_t K) {
          dqt_bwd_dw_img_workspace_size(T, N, K);
 }
 
-size_t dqt_bwd_dw_img_workspace_size(int64_t T, int64_t N, int64_t K) {
+// Slices of a weight gradient, with its update or (update false) written out
+// as it is: one slab of a gradient that is only written out would be the
+// output itself, and launch_gemm uses none.
+static size_t dw_slice_ws(int64_t T, int64_t N, int64_t K, bool update) {
   if (T <= 0 || N <= 0 || K <= 0 || T > kMaxDim || N > kMaxDim || K > kMaxDim) return 0;
   if (dqt::gemm_mode() != 0) return 0;
   const int s = dqt::dw_splits(static_cast<int>(N), static_cast<int>(K), static_cast<int>(T));
+  if (s == 1 && !update) return 0;  // (so few tiles have no last wave to cut)
   if (s > 0) return static_cast<size_t>(s) * static_cast<size_t>(N) * static_cast<size_t>(K) * 4u;
   // last-wave tail: at most one 256 x 256 fp32 slice partial per cluster (at
   // most one cluster per SM pair on any launch)
@@ -571,6 +575,10 @@ size_t dqt_bwd_dw_img_workspace_size(int64_t T, int64_t N, int64_t K) {
       dqt::tail_plan(static_cast<int>(N), static_cast<int>(K), static_cast<int>(T), sms / 2);
   if (tp.splits < 2) return 0;
   return 256 + static_cast<size_t>(sms / 2) * 65536 * sizeof(float);  // + 256: alignment
+}
+
+size_t dqt_bwd_dw_img_workspace_size(int64_t T, int64_t N, int64_t K) {
+  return dw_slice_ws(T, N, K, true);
 }
 
 int dqt_bitlinear_bwd_dw_update(const dqt_bf16* dY, const int8_t* Xq, const float* s_x,
@@ -981,7 +989,7 @@ size_t dqt_bwd_dw_adafactor_workspace_size(int64_t T, int64_t N, int64_t K) {
   if (T <= 0 || N <= 0 || K <= 0 || T > kMaxDim || N > kMaxDim || K > kMaxDim) return 0;
   const size_t g = align256(static_cast<size_t>(N) * static_cast<size_t>(K) * 4u);
   const size_t st = align256(dqt::adafactor_stats_ws(N, K));
-  return g + st + align256(dqt_bwd_dw_img_workspace_size(T, N, K));
+  return g + st + align256(dw_slice_ws(T, N, K, false));
 }
 
 int dqt_bitlinear_bwd_dw_adafactor(const dqt_bf16* dY, const dqt_bf16* Xdq, void* W,

@@ -50,6 +50,20 @@ def test_grid_for_bits(L):
         assert L.dqt_grid_for_bits(C.c_float(bad), C.byref(g)) == dqt.DQT_ERR_ARG
 
 
+def test_adafactor_workspace_holds_no_single_slab(L):
+    """The Adafactor call's GEMM writes its gradient out: one token slice of it
+    is that gradient, so the workspace is the gradient and the statistics, with
+    no slab of its own; several slices have theirs."""
+    def sizes(T, N, K):
+        base = (4 * N * K + 255) // 256 * 256 + (L.dqt_adafactor_workspace_size(N, K) + 255) // 256 * 256
+        return L.dqt_bwd_dw_adafactor_workspace_size(T, N, K) - base, L.dqt_bwd_dw_img_workspace_size(T, N, K)
+    for T, N, K in ((256, 512, 512), (128, 1536, 1536), (8, 16, 16), (4096, 1792, 1792)):
+        extra, slab = sizes(T, N, K)
+        assert slab == 4 * N * K and extra == 0
+    extra, slabs = sizes(4096, 512, 512)
+    assert extra == slabs > 4 * 512 * 512
+
+
 def test_status_strings(L):
     for s in range(6):
         assert L.dqt_status_string(s).startswith(b"DQT")
