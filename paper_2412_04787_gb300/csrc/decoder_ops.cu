@@ -16,6 +16,7 @@
 #include <cuda_bf16.h>
 
 #include "dqt_internal.h"
+#include "per_device.h"
 
 namespace dqt {
 
@@ -601,13 +602,15 @@ static int rms_bwd_launch(const uint16_t* x, const uint16_t* w, const float* rst
                           const uint16_t* dy, int64_t rows, int64_t D, uint16_t* dx,
                           uint16_t* dw, float* part, cudaStream_t stream) {
   auto kern = rmsnorm_bwd_kernel<VPL, WPR>;
-  static bool attr_set = false;  // per template instance
-  if (!attr_set) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             norm_bwd_smem<VPL>()) != cudaSuccess)
-      return 3;
-    attr_set = true;
-  }
+  // the limit on shared memory belongs to a device
+  static PerDevice limit;  // per template instance
+  int dev = 0, set = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || !limit.get(dev, set, [&](int& v) {
+        v = 1;
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    norm_bwd_smem<VPL>()) == cudaSuccess;
+      }))
+    return 3;
   const int64_t blocks = norm_bwd_blocks(rows, D);
   if (launch_dep(kern, static_cast<unsigned>(blocks), 32 * kNormBwdWarps, norm_bwd_smem<VPL>(),
                  stream, reinterpret_cast<const uint4*>(x), reinterpret_cast<const uint4*>(w), rstd,

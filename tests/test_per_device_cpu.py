@@ -1,0 +1,45 @@
+"""The values that the library keeps per device (csrc/per_device.h), on the
+host: a launch attribute set on one device is set on the next one too.  The
+header is compiled as it is, with a stand-in for the CUDA call."""
+import os
+import subprocess
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2412_04787_gb300", "csrc")
+
+
+def _run(tmp_path, body):
+    src, exe = tmp_path / "t.cpp", tmp_path / "t"
+    src.write_text('#include "per_device.h"\n#include <cstdio>\n#include <thread>\n#include <vector>\n'
+                   + body)
+    subprocess.run(["g++", "-std=c++17", "-O1", "-pthread", "-I", CSRC, str(src), "-o", str(exe)],
+                   check=True)
+    return subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()
+
+
+def test_each_device_is_set_once(tmp_path):
+    """One call per device, a failed one is tried again, devices beyond the
+    table are set on each call."""
+    out = _run(tmp_path, """
+      int main() {
+        static dqt::PerDevice p;
+        int calls = 0, v = 0;
+        auto set = [&](int& x) { ++calls; x = 1; return true; };
+        auto fail = [&](int&) { ++calls; return false; };
+        for (int dev : {0, 0, 1, 1, 0, 63, 63}) if (!p.get(dev, v, set) || v != 1) return 1;
+        std::printf("%d ", calls);
+        if (p.get(2, v, fail) || !p.get(2, v, set)) return 1;
+        std::printf("%d ", calls);
+        for (int i = 0; i < 2; ++i) if (!p.get(64, v, set)) return 1;
+        std::printf("%d", calls);
+      }""")
+    assert out == ["3", "5", "7"]
+
+
+def test_launch_attributes_of_the_norm_are_per_device():
+    """The norm's backward needs a raised shared-memory limit, which belongs to
+    a device: no process-wide flag stands before that call."""
+    src = open(os.path.join(CSRC, "decoder_ops.cu")).read()
+    body = src[src.index("static int rms_bwd_launch"):]
+    body = body[:body.index("\n}\n")]
+    assert "static bool" not in body and "PerDevice" in body
