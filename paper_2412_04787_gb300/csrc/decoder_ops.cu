@@ -584,10 +584,12 @@ static int rms_launch(const uint16_t* x, const uint16_t* w, float eps, int64_t r
                       uint16_t* y, float* rstd, cudaStream_t stream) {
   const int nv = static_cast<int>(D / 8);
   // as many blocks as fit at once
-  static int occ = 0;  // per template instance
-  if (occ == 0 && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, rmsnorm_fwd_kernel<VPL>,
-                                                                 32 * kNormWarps, 0) != cudaSuccess ||
-                   occ < 1))
+  static PerDevice per_sm;  // per template instance
+  int dev = 0, occ = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || !per_sm.get(dev, occ, [](int& v) {
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, rmsnorm_fwd_kernel<VPL>,
+                                                             32 * kNormWarps, 0) == cudaSuccess;
+      }))
     occ = 1;
   const int64_t need = (rows + kNormWarps - 1) / kNormWarps;
   const int64_t cap = static_cast<int64_t>(sm_count()) * occ;

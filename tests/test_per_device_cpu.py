@@ -36,6 +36,36 @@ def test_each_device_is_set_once(tmp_path):
     assert out == ["3", "5", "7"]
 
 
+def test_threads_see_whole_values(tmp_path):
+    """A query that writes its result in two steps: no thread reads the first."""
+    out = _run(tmp_path, """
+      int main() {
+        int bad = 0;
+        for (int round = 0; round < 50; ++round) {
+          dqt::PerDevice p;
+          std::atomic<int> wrong{0}, ready{0};
+          std::vector<std::thread> ts;
+          for (int i = 0; i < 4; ++i)
+            ts.emplace_back([&] {
+              ++ready;
+              while (ready.load() < 4) std::this_thread::yield();
+              int v = 0;
+              for (int k = 0; k < 20; ++k)
+                if (!p.get(0, v, [](int& x) { x = -1; std::this_thread::yield(); x = 7; return true; }) || v != 7) ++wrong;
+            });
+          for (auto& t : ts) t.join();
+          bad += wrong;
+        }
+        std::printf("%d", bad);
+      }""")
+    assert out == ["0"]
+
+
+def test_the_norms_occupancy_is_not_queried_into_shared_memory():
+    src = open(os.path.join(CSRC, "decoder_ops.cu")).read()
+    assert "static int occ" not in src
+
+
 def test_launch_attributes_of_the_norm_are_per_device():
     """The norm's backward needs a raised shared-memory limit, which belongs to
     a device: no process-wide flag stands before that call."""
