@@ -35,30 +35,35 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 
 // One 16-byte vector (four pairs of one head) per thread step.  cs holds
 // (cos, sin) per position and pair: fp32 [S, D/2, 2].  A block takes R whole
-// rows side by side (one when a row has as many vectors as the block has
-// threads, or more) and the blocks run through memory in order: the position
-// is a remainder of block indices, and the vector in the head a mask where a
-// head has a power of two of them (head_mask, else -1). Three 64-bit divisions
-// per vector had bound the kernel; two 32-bit remainders per thread still took
-// half of its instructions. 8 x 2048 x 32 x 64 (134 MB): 28.9 -> 23.8 ->
-// 22.5 us.
+// rows (rope_rows), 256 of their vectors at a time, and the blocks run through
+// memory in order: the position is a remainder of block indices, the row in the
+// block a product with 2^31 / row_vecs (row_magic, R > 1; exact while the block's
+// vectors times row_vecs stay below 2^31), and the vector in the head a mask where
+// a head has a power of two of them (head_mask, else -1).
+// Three 64-bit divisions per vector had bound the kernel; two 32-bit remainders
+// per thread still took half of its instructions. 8 x 2048 x 32 x 64 (134 MB):
+// 28.9 -> 23.8 -> 22.5 us.
 template <bool INV>
 __global__ void __launch_bounds__(kRopeThreads)
     rope_kernel(const uint4* __restrict__ x, uint4* __restrict__ y, const float4* __restrict__ cs,
-                int64_t rows, int row_vecs, uint32_t S, int head_vecs, int head_mask,
-                int R) {
+                int64_t rows, int row_vecs, uint32_t S, int head_vecs, int head_mask, int R,
+                uint32_t row_magic) {
   dep_wait();
-  const int tr = row_vecs < kRopeThreads ? static_cast<int>(threadIdx.x) / row_vecs : 0;
-  const int64_t row = static_cast<int64_t>(blockIdx.x) * R + tr;
-  if (tr >= R || row >= rows) return;
-  // the position: a remainder of block indices, then tr steps
-  uint32_t pos = (blockIdx.x * static_cast<uint32_t>(R)) % S + static_cast<uint32_t>(tr);
-  if (pos >= S) pos = pos - S < S ? pos - S : pos % S;
-  const float4* table = cs + static_cast<int64_t>(pos) * head_vecs * 2;
-  for (int v = static_cast<int>(threadIdx.x) - tr * row_vecs; v < row_vecs; v += kRopeThreads) {
+  const int64_t row0 = static_cast<int64_t>(blockIdx.x) * R;
+  const int n = static_cast<int>(rows - row0 < R ? rows - row0 : R) * row_vecs;
+  const uint32_t pos0 = (blockIdx.x * static_cast<uint32_t>(R)) % S;
+  x += row0 * row_vecs;
+  y += row0 * row_vecs;
+#pragma unroll 1
+  for (int l = threadIdx.x; l < n; l += kRopeThreads) {
+    const uint4 xv = __ldcs(x + l);
+    const int r = R > 1 ? static_cast<int>(__umulhi(2u * static_cast<uint32_t>(l), row_magic)) : 0;
+    const int v = l - r * row_vecs;
+    uint32_t pos = pos0 + static_cast<uint32_t>(r);
+    if (pos >= S) pos = pos - S < S ? pos - S : pos % S;
     // four pairs = eight floats = two float4 of the table
-    const float4* t = table + 2 * (head_mask >= 0 ? v & head_mask : v % head_vecs);
-    const uint4 xv = __ldcs(x + row * row_vecs + v);
+    const float4* t = cs + 2 * (static_cast<int64_t>(pos) * head_vecs +
+                                (head_mask >= 0 ? v & head_mask : v % head_vecs));
     const float4 c01 = __ldg(t), c23 = __ldg(t + 1);
     const float cth[4] = {c01.x, c01.z, c23.x, c23.z};
     const float sth[4] = {INV ? -c01.y : c01.y, INV ? -c01.w : c01.w, INV ? -c23.y : c23.y,
@@ -72,7 +77,7 @@ __global__ void __launch_bounds__(kRopeThreads)
       const float yo = __fadd_rn(__fmul_rn(xe, sth[j]), __fmul_rn(xo, cth[j]));
       o[j] = pack_bf16x2(ye, yo);
     }
-    y[row * row_vecs + v] = make_uint4(o[0], o[1], o[2], o[3]);
+    y[l] = make_uint4(o[0], o[1], o[2], o[3]);
   }
 }
 
@@ -515,20 +520,41 @@ unsigned grid_full(int64_t items, int threads) {
   return static_cast<unsigned>(b < 1 ? 1 : b < most ? b : most);
 }
 
+// Rows per block of the rotary embedding: as many as 256 threads hold, or, where
+// that leaves more than a sixteenth of the threads idle, the count of at most
+// 2048 vectors that leaves the fewest, as long as every SM still gets four
+// blocks.  With one row per block at 136 vectors a row (8 x 2048 x 17 x 64, 71
+// MB) half of the threads had nothing to do: 18.1 us, 13.5 so (15.6 with the
+// divisions); at 264 (4 x 2048 x 33 x 64) 16.0 and 13.2 (15.3), with up to 4096
+// vectors 15.1.
+int rope_rows(int row_vecs, int64_t rows) {
+  int R = row_vecs < kRopeThreads ? kRopeThreads / row_vecs : 1;
+  const auto idle = [&](int64_t r) {
+    const int64_t v = r * row_vecs, t = (v + kRopeThreads - 1) / kRopeThreads * kRopeThreads;
+    return static_cast<double>(t - v) / static_cast<double>(t);
+  };
+  if (idle(R) <= 1.0 / 16) return R;
+  const int64_t most = rows / (4 * sm_count());
+  for (int64_t r = R + 1; r <= most && r * row_vecs <= 2048; ++r)
+    if (idle(r) < idle(R) - 1.0 / 64) R = static_cast<int>(r);
+  return R;
+}
+
 }  // namespace
 
 int launch_rope(const uint16_t* x, uint16_t* y, const float* cos_sin, int64_t rows, int64_t S,
                 int64_t H, int64_t D, bool inverse, cudaStream_t stream) {
   // H D < 2^31 and S < 2^31 (checked by the caller): 32-bit columns and positions
   const int row_vecs = static_cast<int>(H * D / 8), head_vecs = static_cast<int>(D / 8);
-  const int R = row_vecs < kRopeThreads ? kRopeThreads / row_vecs : 1;
+  const int R = rope_rows(row_vecs, rows);
   const unsigned blocks = static_cast<unsigned>((rows + R - 1) / R);
+  const uint32_t magic = static_cast<uint32_t>((int64_t(1) << 31) / row_vecs + 1);
   auto* xv = reinterpret_cast<const uint4*>(x);
   auto* yv = reinterpret_cast<uint4*>(y);
   auto* cv = reinterpret_cast<const float4*>(cos_sin);
   return launch_dep(inverse ? rope_kernel<true> : rope_kernel<false>, blocks, kRopeThreads, 0,
                     stream, xv, yv, cv, rows, row_vecs, static_cast<uint32_t>(S), head_vecs,
-                    (head_vecs & (head_vecs - 1)) == 0 ? head_vecs - 1 : -1, R);
+                    (head_vecs & (head_vecs - 1)) == 0 ? head_vecs - 1 : -1, R, magic);
 }
 
 int launch_ce_fwd(const uint16_t* logits, const int64_t* targets, int64_t M, int64_t V,

@@ -56,6 +56,19 @@ def test_rope_matches_fp32_formula(B, S, H, D):
     assert (back - x.float()).abs().max() <= 2 ** -7 * x.float().abs().max()
 
 
+# rows of 1 vector (a block has 256 of them), 136, 168, 264 and 288 vectors (a
+# block takes several rows in steps of 256 vectors), with positions that come
+# round again within a block and a last block that is not full
+@pytest.mark.parametrize("B,S,H,D", [(3, 5, 1, 8), (2100, 3, 17, 64), (1, 9151, 17, 64),
+                                     (5, 1001, 21, 64), (5, 2001, 33, 64), (2, 3001, 32, 72)])
+def test_rope_rows_per_block(B, S, H, D):
+    x = inputs.normal((B, S, H, D), 1.0, seed=S, dtype=torch.bfloat16).cuda()
+    ang = torch.arange(S * (D // 2), dtype=torch.float32).view(S, D // 2) * 0.37
+    cs = torch.stack((ang.cos(), ang.sin()), -1).contiguous().cuda()
+    assert torch.equal(dqt.dqt_rope_bf16(x, cs), _rope_ref(x, cs))
+    assert torch.equal(dqt.dqt_rope_bf16(x, cs, inverse=True), _rope_ref(x, cs, -1.0))
+
+
 def test_rope_backward_is_the_transpose():
     from paper_2412_04787_gb300.decoder import _Rope
     B, S, H, D = 2, 24, 4, 64
