@@ -331,8 +331,9 @@ __global__ void __launch_bounds__(32 * kNormWarps)
 //   dw_j = sum over rows of dy_j x_j r
 // A row is taken by WPR warps (two beyond D = 1024, so that a lane's dw sums
 // leave registers for sixteen warps per SM: with eight the kernel waited on
-// its own arithmetic), VPL vectors per lane.  Each group walks rows group,
-// group + groups, ..., the next kNormStages - 1 rows on their way into shared
+// its own arithmetic), VPL vectors per lane.  A block has its groups on rows that
+// follow one another, or (spread, for few rows) one on a row in turn with the
+// other blocks.  Each group walks rows group, group + groups, ..., the next kNormStages - 1 rows on their way into shared
 // memory while the current one is reduced (each lane copies the vectors that
 // it reads itself), and keeps its dw partial sums in registers; at the end the
 // block's groups add theirs in order in shared memory and write one partial
@@ -360,7 +361,7 @@ template <int VPL, int WPR>
 __global__ void __launch_bounds__(32 * kNormBwdWarps, 1)
     rmsnorm_bwd_kernel(const uint4* __restrict__ x, const uint4* __restrict__ w,
                        const float* __restrict__ rstd, const uint4* __restrict__ dy, int64_t rows,
-                       int nv, uint4* __restrict__ dx, float* __restrict__ part) {
+                       int nv, bool spread, uint4* __restrict__ dx, float* __restrict__ part) {
   dep_wait();
   constexpr int G = kNormBwdWarps / WPR;       // row groups per block
   __shared__ float4 sums[VPL * WPR * 64];      // one row of columns
@@ -369,13 +370,14 @@ __global__ void __launch_bounds__(32 * kNormBwdWarps, 1)
   extern __shared__ uint4 norm_ring[];         // [warp][stage][x, dy][VPL * 32]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int grp = warp / WPR, sub = warp % WPR;
-  const int64_t gid = static_cast<int64_t>(blockIdx.x) * G + grp;
+  // the groups' first rows: gid0, gid0 + gstep, ...
+  const int64_t gid0 = spread ? blockIdx.x : static_cast<int64_t>(blockIdx.x) * G;
+  const int64_t gstep = spread ? gridDim.x : 1;
+  const int64_t gid = gid0 + grp * gstep;
   const int64_t ngrp = static_cast<int64_t>(gridDim.x) * G;
   const float inv_d = 1.0f / static_cast<float>(nv * 8);
   uint4* ring = norm_ring + warp * (kNormStages * 2 * VPL * 32);
   const int c0 = sub * 32 + lane;  // vector k of this lane: column c0 + 32 WPR k
-  for (int i = threadIdx.x; i < nv; i += 32 * kNormBwdWarps) gain[i] = __ldg(w + i);
-  __syncthreads();
   float acc[VPL][8];
 #pragma unroll
   for (int k = 0; k < VPL; ++k)
@@ -396,6 +398,8 @@ __global__ void __launch_bounds__(32 * kNormBwdWarps, 1)
 #pragma unroll
   for (int i = 0; i < kNormStages - 1; ++i) load(gid + i * ngrp, i);
   float rn = gid < rows ? rstd[gid] : 0.0f;
+  for (int i = threadIdx.x; i < nv; i += 32 * kNormBwdWarps) gain[i] = __ldg(w + i);
+  __syncthreads();
   int stage = 0, turn = 0;
   for (int64_t row = gid; row < rows; row += ngrp) {
     const float r = rn;
@@ -454,8 +458,9 @@ __global__ void __launch_bounds__(32 * kNormBwdWarps, 1)
       __stcs(dx + row * nv + c, make_uint4(o[0], o[1], o[2], o[3]));
     }
   }
-  // the block's sum, its groups in order
-  for (int t = 0; t < G; ++t) {
+  // the block's sum, its groups that had rows in order (a loop of its own for
+  // all G: unrolled, it costs 0.3 us less)
+  auto add = [&](int t) {
     if (grp == t) {
 #pragma unroll
       for (int k = 0; k < VPL; ++k) {
@@ -473,6 +478,11 @@ __global__ void __launch_bounds__(32 * kNormBwdWarps, 1)
       }
     }
     __syncthreads();
+  };
+  if (gid0 + (G - 1) * gstep < rows) {
+    for (int t = 0; t < G; ++t) add(t);
+  } else {
+    for (int t = 0; gid0 + t * gstep < rows; ++t) add(t);
   }
   float4* pr = reinterpret_cast<float4*>(part + static_cast<int64_t>(blockIdx.x) * nv * 8);
   for (int i = threadIdx.x; i < 2 * nv; i += 32 * kNormBwdWarps) pr[i] = sums[i];
@@ -593,11 +603,20 @@ int launch_swiglu_bwd(const uint16_t* g, const uint16_t* u, const uint16_t* dh, 
                     reinterpret_cast<uint4*>(du), nvec);
 }
 
-// Warps per row of the backward, and its blocks: one per SM at most.
+// Warps per row of the backward, and its blocks: one per SM at most.  Few rows
+// (half of what the SMs' row groups hold) are spread over the SMs, one group of
+// each block after the other: a block that held sixteen of them added sixteen
+// gain sums in turn (16 x 1000: 8.5 us, 3.8 so; 1000 x 1000 9.3 and 6.7), while
+// rows in block order suit the memory better (16384 x 1000: 20.6 us, spread
+// 22.3).
 static int norm_bwd_wpr(int64_t D) { return D > 1024 ? 2 : 1; }
+static bool norm_bwd_spread(int64_t rows, int64_t D) {
+  return 2 * rows <= static_cast<int64_t>(sm_count()) * (kNormBwdWarps / norm_bwd_wpr(D));
+}
 static int64_t norm_bwd_blocks(int64_t rows, int64_t D) {
   const int64_t per_block = kNormBwdWarps / norm_bwd_wpr(D);
-  const int64_t need = (rows + per_block - 1) / per_block, sms = sm_count();
+  const int64_t need = norm_bwd_spread(rows, D) ? rows : (rows + per_block - 1) / per_block;
+  const int64_t sms = sm_count();
   return sms < need ? sms : need;
 }
 
@@ -643,7 +662,7 @@ static int rms_bwd_launch(const uint16_t* x, const uint16_t* w, const float* rst
   if (launch_dep(kern, static_cast<unsigned>(blocks), 32 * kNormBwdWarps, norm_bwd_smem<VPL>(),
                  stream, reinterpret_cast<const uint4*>(x), reinterpret_cast<const uint4*>(w), rstd,
                  reinterpret_cast<const uint4*>(dy), rows, static_cast<int>(D / 8),
-                 reinterpret_cast<uint4*>(dx), part))
+                 norm_bwd_spread(rows, D), reinterpret_cast<uint4*>(dx), part))
     return 3;
   return launch_dep(rmsnorm_dw_kernel, static_cast<unsigned>((D + 31) / 32), 1024, 0, stream, part,
                     blocks, static_cast<int>(D), dw);

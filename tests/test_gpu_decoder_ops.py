@@ -174,6 +174,15 @@ def test_rmsnorm_matches_fp64(rows, D):
     assert ((y.float() - ref_t.float()).abs() <= 2 ** -6 * ref_t.float().abs() + 1e-6).all()
 
 
+# few rows: a block per row, several row groups of each block (up to 1216 rows
+# on 152 SMs, 608 of more than 1024 columns), whole blocks beyond, with a last
+# block that has fewer rows
+@pytest.mark.parametrize("rows,D", [(2, 1000), (16, 1032), (151, 264), (153, 2048), (608, 1536), (609, 1536),
+                                    (1000, 1032), (1216, 1024), (1217, 1024), (2433, 8), (2431, 512)])
+def test_rmsnorm_rows_over_blocks(rows, D):
+    test_rmsnorm_matches_fp64(rows, D)
+
+
 def test_rmsnorm_gain_gradient_is_deterministic():
     from paper_2412_04787_gb300.decoder import _RMSNorm
     x = inputs.normal((4096, 768), 1.0, seed=9, dtype=torch.bfloat16).cuda()
