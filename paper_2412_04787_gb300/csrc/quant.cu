@@ -9,10 +9,10 @@
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
 
-#include <numeric>
 #include <type_traits>
 
 #include "dqt_internal.h"
+#include "ring_geometry.h"
 
 namespace dqt {
 
@@ -202,10 +202,10 @@ __global__ void __launch_bounds__(kAqWarps * 32)
 // 1 reduces amax over the row in shared memory, pass 2 re-reads it and writes
 // the outputs.  Every slot carries a `full` barrier (the copy's bytes) and an
 // `empty` barrier (an arrive per row); the ring keeps up to 192 KB of rows in
-// flight per SM, which a register-held design cannot.  With both images 16384
-// x 768 takes 12.5 us (16.8 with whole chunks per warp and a table of
-// quotients per row), 256 x 512 2.1 (3.9), 8192 x 2048 13.5 (15.0); the codes
-// alone 11.5 (10.9) there, 21.5 (23.3) at 8192 x 5632.
+// flight per SM, which a register-held design cannot (ring_geometry.h).  With
+// both images 16384 x 768 takes 10.9 us (16.8 with whole chunks per warp and a
+// table of quotients per row), 256 x 512 2.1 (3.9), 8192 x 2048 12.0 (15.0); the
+// codes alone 10.3 (10.9) there, 21.8 (23.3) at 8192 x 5632.
 //
 // amax is reduced on pairs of bf16 magnitudes (max.bf16x2 returns the
 // non-NaN operand, as fmaxf does, and is exact).  Round(y) for the int8
@@ -216,9 +216,6 @@ __global__ void __launch_bounds__(kAqWarps * 32)
 // 127 + 2^-17 and the sum never exceeds 1.5 * 2^23 + 127: only the lower
 // clamp is needed, and it maps a NaN product (an infinite input) to -128, as
 // act_quant_kernel does.
-constexpr int kAqbRing = 192 * 1024;  // shared-memory bytes of the row ring
-constexpr int kRingWarps = 24;        // consumer warps at most
-
 // Linear bulk copy (no tensor map) of `bytes` from global memory into this
 // CTA's shared memory, completing on `bar`, whose expected byte count the
 // caller has raised by `bytes`.  Both addresses 16-byte aligned; `bytes` a
@@ -718,33 +715,13 @@ int grid_for(int64_t work, int threads) {
 
 namespace {
 
-// Geometry of a row ring (act_quant_bulk_kernel, codes_to_xdq_bulk_kernel):
-// chunks of about 8 KB (rows of up to 8 KB are copied one per chunk), then as
-// many slots as fit in kAqbRing bytes (48 at most) and up to max_warps consumer
-// warps; false when fewer than four chunks fit.  One producer thread issues a
-// bulk copy about every 0.2 us whatever its size, so copies below ~8 KB leave
-// the ring short of bytes in flight.
-//
-// S rpc is a multiple of W: the row that a warp waits for and the one that used
-// the same place of the ring before, S rpc rows earlier, are then the same
-// warp's.  A warp that could reach a slot before the slot's previous chunk had
-// landed would wait on a phase parity that reads as complete.
-bool ring_geometry(int64_t row_bytes, int max_warps, int& rpc, int& W, int& S) {
-  rpc = row_bytes >= 8192 ? 1 : static_cast<int>(8192 / row_bytes);
-  const int64_t fit = kAqbRing / (rpc * row_bytes);
-  if (fit < 4) return false;
-  const int smax = static_cast<int>(fit < 48 ? fit : 48);
-  S = W = 0;
-  for (int w = max_warps < smax * rpc ? max_warps : smax * rpc; w > 0; --w) {
-    const int unit = w / std::gcd(w, rpc);  // S is a multiple of it
-    const int s = smax / unit * unit;
-    if (w * s > W * S) {
-      W = w;
-      S = s;
-    }
-  }
-  return true;
+int sm_count() {
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
 }
+
 constexpr int kRingMaxSmem = kAqbRing + 16 * 48 + 512 * kRingWarps;  // ring, barriers, tables
 
 // Launches a row-ring kernel: one CTA per SM (at most T), 32 (W + 1) threads.
@@ -759,10 +736,7 @@ int launch_ring(Kern kern, bool& attr_set, bool tables, int64_t T, int rpc, int 
   }
   unsigned int* status = status_word();
   if (!status) return 3;
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int blocks = static_cast<int>(T < sms ? T : sms);
+  const int sms = sm_count(), blocks = static_cast<int>(T < sms ? T : sms);
   const size_t smem = static_cast<size_t>(S) * rpc * row_bytes + 16 * static_cast<size_t>(S) +
                       (tables ? 512 * W : 0);
   return launch_dep(kern, blocks, 32 * (W + 1), smem, stream, args..., S, W, rpc, status,
@@ -775,7 +749,9 @@ template <bool F8, bool IMG, int XDQ>
 int launch_aq_ring(const uint16_t* X, int64_t T, int64_t K, int8_t* Xq, float* s_x,
                    uint16_t* Xq_img, uint16_t* Xdq, cudaStream_t stream) {
   int rpc, W, S;
-  if (!ring_geometry(2 * K, kRingWarps, rpc, W, S)) return -1;
+  constexpr RingKind kind = F8 ? (XDQ ? RING_E4M3_XDQ : RING_E4M3)
+                               : (IMG || XDQ ? RING_IMAGES : RING_CODES);
+  if (!ring_geometry(2 * K, ring_bytes(kind, T, K, sm_count()), rpc, W, S)) return -1;
   static bool attr_set = false;  // per template instance
   return launch_ring(act_quant_bulk_kernel<F8, IMG, XDQ>, attr_set, XDQ == 2, T, rpc, W, S, 2 * K,
                      stream, X, static_cast<int>(T), static_cast<int>(K), Xq, s_x, Xq_img, Xdq);
@@ -819,7 +795,7 @@ int launch_codes_to_xdq(const int8_t* Xq, const float* s_x, int64_t T, int64_t K
                         cudaStream_t stream) {
   {
     int rpc, W, S;
-    if (ring_geometry(K, kRingWarps, rpc, W, S)) {
+    if (ring_geometry(K, ring_bytes(RING_XDQ, T, K, sm_count()), rpc, W, S)) {
       static bool attr_set = false;
       return launch_ring(codes_to_xdq_bulk_kernel, attr_set, false, T, rpc, W, S, K, stream, Xq, s_x,
                          static_cast<int>(T), static_cast<int>(K), Xdq);

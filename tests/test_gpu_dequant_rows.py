@@ -84,3 +84,21 @@ def test_row_ring_many_rounds(T, K):
     assert torch.equal(first[1], s.float())
     want = (x.float() * first[1][:, None]).round().clamp_(-128, 127)
     assert torch.equal(first[0].float(), want)
+
+
+@pytest.mark.parametrize("T,K", [(8192, 2048), (8192, 4096), (16384, 768), (16384, 3584), (8192, 5632),
+                                 (16384, 272), (4096, 8192), (3000, 1040)])
+def test_each_output_alone(T, K):
+    """Codes, code image and X_tilde written alone, and E4M3 codes alone: rings
+    of other sizes than the call that writes all outputs has, the same bytes."""
+    x = torch.randn(T, K, generator=torch.Generator().manual_seed(T + K)).to(torch.bfloat16).cuda()
+    q, s, img, xdq = dqt.dqt_act_quant_images(x)
+    q8, s8, _ = dqt.dqt_act_quant_fp8(x)
+    for _ in range(20):
+        a, sa = dqt.dqt_act_quant(x)
+        assert torch.equal(a, q) and torch.equal(sa, s)
+        assert torch.equal(dqt.dqt_act_quant_images(x, want=("Xq_img",))[2], img)
+        assert torch.equal(dqt.dqt_act_quant_images(x, want=("Xdq",))[3], xdq)
+        b, sb, none = dqt.dqt_act_quant_fp8(x, want_xdq=False)
+        assert none is None and torch.equal(b, q8) and torch.equal(sb, s8)
+    dqt.dqt_check_device_status()
