@@ -16,7 +16,6 @@
 #include <cuda_bf16.h>
 
 #include "dqt_internal.h"
-#include "per_device.h"
 
 namespace dqt {
 
@@ -512,13 +511,6 @@ __global__ void __launch_bounds__(1024)
     const __nv_bfloat16 h = __float2bfloat16_rn(t);
     dw[col] = *reinterpret_cast<const uint16_t*>(&h);
   }
-}
-
-int sm_count() {
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms;
 }
 
 // One item per thread, blocks in memory order: a grid of the resident blocks

@@ -7,6 +7,7 @@
 
 #include "../../include/dqt.h"
 #include "dqt_device.cuh"
+#include "per_device.h"
 
 namespace dqt {
 
@@ -45,6 +46,17 @@ int launch_dep(void (*kern)(KArgs...), dim3 grid, unsigned threads, size_t smem,
   cfg.numAttrs = 1;
   if (cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...) != cudaSuccess) return 3;
   return cudaPeekAtLastError() == cudaSuccess ? 0 : 3;
+}
+
+// SMs of the current device (148 without one).
+inline int sm_count() {
+  static PerDevice kept;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || !kept.get(dev, sms, [&](int& n) {
+        return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+      }))
+    return 148;
+  return sms;
 }
 
 // GEMM kernel selection: 0 = 2-SM pair tiles where possible, 1 = 1-SM tiles.

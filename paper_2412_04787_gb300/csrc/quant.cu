@@ -715,13 +715,6 @@ int grid_for(int64_t work, int threads) {
 
 namespace {
 
-int sm_count() {
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms;
-}
-
 constexpr int kRingMaxSmem = kAqbRing + 16 * 48 + 512 * kRingWarps;  // ring, barriers, tables
 
 // Launches a row-ring kernel: one CTA per SM (at most T), 32 (W + 1) threads.

@@ -145,3 +145,40 @@ def test_four_streams_equal_one_stream():
         assert torch.equal(a[key], b[key]), key
     # the steps did change codes (the comparison is not of untouched state)
     assert all(int(serial[name]["changed"].item()) > 0 for name, _, _ in PROJ)
+
+
+def test_captured_four_streams_equal_one_stream():
+    """The same step captured over the four streams and replayed (a captured
+    library launch is tied to its stream's previous one by a programmatic edge,
+    and to the other streams' by full ones): new inputs for each replay, and the
+    bytes of eager launches on one stream.  Before the forward of gate and of up
+    two library streams join, and four before the down projection."""
+    serial, replayed = _state(), _state()
+    streams = [torch.cuda.Stream() for _ in range(4)]
+
+    def load(st, seed):
+        st["X"].copy_(inputs.normal((T, H), 1.0, seed=seed, dtype=torch.bfloat16))
+        st["H"].copy_(inputs.normal((T, I), 1.0, seed=seed + 1, dtype=torch.bfloat16))
+        for i, (name, _, N) in enumerate(PROJ):
+            st[name]["dY"].copy_(inputs.normal((T, N), 1e-2, seed=seed + 2 + i, dtype=torch.bfloat16))
+
+    _step(_state(), streams)  # first calls of a process set kernels up
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        _step(replayed, streams)
+    one = torch.cuda.current_stream()
+    for replay in range(4):
+        load(serial, 100 + 10 * replay)
+        load(replayed, 100 + 10 * replay)
+        for name, _, _ in PROJ:
+            for key in ("Y", "dX"):
+                replayed[name][key].fill_(float("nan"))
+        _step(serial, [one] * 4)
+        graph.replay()
+        torch.cuda.synchronize()
+        dqt.dqt_check_device_status()
+        a, b = _snapshot(serial), _snapshot(replayed)
+        for key in a:
+            assert torch.equal(a[key], b[key]), (replay, key)
+    assert all(int(serial[name]["changed"].item()) > 0 for name, _, _ in PROJ)
