@@ -94,7 +94,8 @@ DW_TRAFFIC_STACKED = {"e8a6edbac357": ((499344640 + 147830784)
                                          + (259118848 + 57005568 + 33063680 + 768)) // 2}
 # DRAM bytes (read + write, ncu) of the grouped launch of both dW problems
 DW_TRAFFIC_GROUP = {"7eaccd5d9509": 873590272 + 328523520,
-                    "b4d7fef19bff": 820908288 + 328113920}
+                    "b4d7fef19bff": 820908288 + 328113920,
+                    "0b28b7d25826": 804748800 + 328048896}
 DW_TRAFFIC_BYTES = {"ac36c0aa63c5": 261135360 + 57050112 + 33049600,
                     "82d12725fdfa": 262571008 + 61169152 + 33047808,
                     "a25cf8632190": 261430272 + 59386112 + 33048064}

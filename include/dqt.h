@@ -627,8 +627,8 @@ int dqt_rmsnorm_bf16(const dqt_bf16* x, const dqt_bf16* w, float eps, int64_t ro
 /* Its backward for the upstream gradient dy [rows, D]:
  *   dx_j = rstd w_j dy_j - x_j rstd^3 (1/D) sum_k w_k dy_k x_k   (bf16 [rows, D])
  *   dw_j = sum over rows of dy_j x_j rstd                        (bf16 [D])
- * dw is summed in a fixed order (per-warp partial sums in the workspace, then
- * a column reduction), so it is deterministic.  Workspace:
+ * dw is summed in a fixed order (one partial row per block in the workspace,
+ * then a column reduction), so it is deterministic.  Workspace:
  * dqt_rmsnorm_bwd_workspace_size(rows, D) bytes for the current device,
  * 16-byte aligned. */
 size_t dqt_rmsnorm_bwd_workspace_size(int64_t rows, int64_t D);

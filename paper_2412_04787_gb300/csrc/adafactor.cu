@@ -3,7 +3,8 @@
 // ICML 2018).  The second moment of an N x K gradient G is kept factored as
 // its row means R [N] and column means C [K]; there is no first moment and no
 // per-weight optimiser state, so a step reads G and the codes and writes the
-// codes.  Four launches, each HBM-bound or tiny:
+// codes.  Four launches: two passes over G bound by HBM, a short one between
+// them, and the element step, bound by instruction issue (af_apply_kernel):
 //
 //   af_sq_partials  one read of G (and the codes): per 128-column chunk row
 //                   sums and per row slab column sums of g^2 + eps1, and the
@@ -360,7 +361,8 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // Rows per block of the two passes over the gradient: halved while the grid
-// is below two blocks per SM (152), each block then having fewer rounds of
+// is below 304 blocks, two per SM of a GB300 (a constant: the rows set the order
+// of the column sums, which is then the same on every device), each block then having fewer rounds of
 // loads to wait for (statistics of 2048 x 768: 22.5 -> 17.0 us, of 512 x 512:
 // 20.6 -> 15.7; where 32 rows give more blocks, 16 are no faster: 27.6 against
 // 28.0 us at 5632 x 2048, 32.1 against 30.9 at 2048 x 5632).  The column sums'

@@ -11,8 +11,8 @@
 //   ce_bwd_kernel    dx_v = (exp(x_v - lse) - [v == target]) * scale
 //   swiglu_kernel    h = silu(g) u, and its backward dg, du
 //   rmsnorm_*        y = x rstd w with rstd = 1 / sqrt(mean(x^2) + eps) per
-//                    row, and its backward (dx per row; dw as per-warp partial
-//                    sums reduced in a fixed order)
+//                    row, and its backward (dx per row; dw as one partial row
+//                    per block, added up in a fixed order)
 #include <cuda_bf16.h>
 
 #include "dqt_internal.h"

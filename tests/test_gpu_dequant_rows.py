@@ -66,8 +66,8 @@ def test_codes_to_xdq_at_extreme_scales(s):
 @pytest.mark.parametrize("T,K", [(8192, 5632), (16384, 768), (8192, 2048), (8192, 1040), (4096, 4112), (8192, 4096),
                                  (8192, 3584)])
 def test_row_ring_many_rounds(T, K):
-    """Many rounds of the shared-memory row ring (each slot refilled up to ten
-    times), launched again and again: a warp that took a slot's old rows, or
+    """Several rounds of the shared-memory row ring (each place of it used up to
+    five times), launched again and again: a warp that took a slot's old rows, or
     released a slot early, would change bytes or run into a wait's limit."""
     x = torch.randn(T, K, generator=torch.Generator().manual_seed(K)).to(torch.bfloat16).cuda()
     first = None
